@@ -164,6 +164,7 @@ void for_each_buffer(const pmr_config& cfg, pmr_ctx* c, F alloc) {
         alloc((void**)(c ? &c->nn_y : nullptr), sizeof(float) * N3);
         alloc((void**)(c ? &c->nn_m1 : nullptr), sizeof(uint16_t) * 4 * N3);
         alloc((void**)(c ? &c->nn_m2 : nullptr), sizeof(uint8_t) * 4 * N3);
+        if (cfg.head == 1) alloc((void**)(c ? &c->nn_mass : nullptr), sizeof(float) * N3);
     }
     alloc((void**)(c ? &c->cA : nullptr), sizeof(float2) * NH);
     alloc((void**)(c ? &c->cB : nullptr), sizeof(float2) * NH);

@@ -208,6 +208,7 @@ struct pmr_ctx {
     float* nn_y = nullptr;      // tensor-core network forward, saved per voxel for its backward: y [N3],
     uint16_t* nn_m1 = nullptr;  // layer-1 ReLU mask [4][N3] (16 columns each),
     uint8_t* nn_m2 = nullptr;   // layer-2 ReLU mask [4][N3] (8 columns each)
+    float* nn_mass = nullptr;   // output of the mass network [N3] (two-network head)
     float2* cA = nullptr;   // complex work arrays, NH each
     float2* cB = nullptr;
     float2* c3 = nullptr;   // 3 * NH
@@ -319,7 +320,8 @@ void mlp_tc_free(pmr_ctx* c);
 int mlp_tc_forward(pmr_ctx* c, const float* feat, float* M, int nsplit, float a);
 int mlp_tc_backward_gv(pmr_ctx* c, const float* feat, const float* gM, int nsplit, float a);  // -> c->gbox
 int mlp_tc_box_floats(int N);               // size of c->gbox
-int stencil_tiles(pmr_ctx* c, float* gfeat);  // c->gbox -> input gradient of the three fields
+// c->gbox (+ the mass network's part) -> input gradient of the three fields
+int stencil_tiles(pmr_ctx* c, const float* feat, const float* gM, float a, float* gfeat);
 
 // loss (loss.cu) ----------------------------------------------------------------
 int residual_forward(pmr_ctx* c, const float* data, const pmr_anneal* an, double* L_res_dev);

@@ -61,8 +61,7 @@ constexpr int HALO = 3 * HX * HY * HZ;
 // TMEM columns of the forward: D1 buffers at COL_D1 and COL_D1 + 64, D2 at COL_D2
 constexpr uint32_t COL_D1 = 0, COL_D2 = 128;
 
-constexpr uint32_t VEC_MASS = 160;  // float offset of the mass-network weights in the vector block
-constexpr uint32_t SZ_VEC = 1920;    // b1[64], b2[32], w3[32], b3[4], mass network[301]: 4 * 461 rounded to 128 B
+constexpr uint32_t SZ_VEC = 640;  // b1[64], b2[32], w3[32], b3[4]: 4 * 132 rounded to 128 B
 
 // Layer 1 of the forward runs on z-line tiles: 128 voxels (x, y, z0 .. z0+127)
 // of one line along z. Its operand image holds, for rows i = 0 .. ZR-1 (the
@@ -280,12 +279,88 @@ struct TileMap {
 };
 
 // Saved activations of the forward: y[N3], layer-1 mask m1[4][N3] (16 bits per
-// column block), layer-2 mask m2[4][N3] (8 bits per column block).
+// column block), layer-2 mask m2[4][N3] (8 bits per column block); with the
+// two-network head also the mass network's output mass[N3] (k_mass_fwd).
 struct Saved {
     float* y;
     uint16_t* m1;
     uint8_t* m2;
+    float* mass;
 };
+
+// ----------------------------------------------------------------------------- mass network
+//
+// The two-network head's mass network (3 -> 20 -> 10 -> 1, ELU) reads the voxel's
+// own three fields only, so it runs outside the tensor-core kernels, one voxel a
+// thread, fully unrolled: every weight is a constant operand of its FMA (kernel
+// parameter space) and all 30 units stay in registers. It is bound by instruction
+// issue (the 30 exponentials take most of it). Inside the tensor-core kernels one
+// compute thread in four evaluated it from shared-memory weights while the rest of
+// its tile waited, which cost more than the trunk: at 192^3 the forward went
+// 2.95 -> 1.32 ms + 0.29 ms (k_mass_fwd) and the backward 3.86 + 0.14 ms ->
+// 1.09 + 0.50 ms (k_stencil_tiles with the mass network's gradient).
+struct MassW {
+    float w[kMassWeights];
+};
+
+// h = ELU(Wm1 f + bm1)
+__device__ __forceinline__ void mass_hidden1(const MassW& W, float f0, float f1, float f2, float (&h)[20]) {
+#pragma unroll
+    for (int j = 0; j < 20; ++j)
+        h[j] = elu_f(W.w[60 + j] + W.w[3 * j] * f0 + W.w[3 * j + 1] * f1 + W.w[3 * j + 2] * f2);
+}
+
+// pre-activations of the second hidden layer
+__device__ __forceinline__ void mass_hidden2(const MassW& W, const float (&h)[20], float (&p2)[10]) {
+#pragma unroll
+    for (int i = 0; i < 10; ++i) {
+        p2[i] = W.w[280 + i];
+#pragma unroll
+        for (int j = 0; j < 20; ++j) p2[i] = fmaf(W.w[80 + 20 * i + j], h[j], p2[i]);
+    }
+}
+
+constexpr int kMassT = 256;
+
+// mass = m, M = M_scale sigmoid(a y) m from the trunk's y
+__global__ void __launch_bounds__(kMassT) k_mass_fwd(const __grid_constant__ MassW W, const float* __restrict__ feat,
+                                                     const float* __restrict__ y, int64_t N3, float M_scale, float a,
+                                                     float* __restrict__ mass, float* __restrict__ M) {
+    const int64_t v = (int64_t)blockIdx.x * kMassT + threadIdx.x;
+    if (v >= N3) return;
+    float h[20], p2[10];
+    mass_hidden1(W, feat[v], feat[N3 + v], feat[2 * N3 + v], h);
+    mass_hidden2(W, h, p2);
+    float m = W.w[300];
+#pragma unroll
+    for (int i = 0; i < 10; ++i) m = fmaf(W.w[290 + i], elu_f(p2[i]), m);
+    mass[v] = m;
+    M[v] = M_scale * sigmoidf(a * y[v]) * m;
+}
+
+// g_c += gm dm/df_c at (f0, f1, f2). The ELU's slope is 1 for x > 0 and e^x =
+// ELU(x) + 1 otherwise, so no second exponential is taken.
+__device__ __forceinline__ void mass_grad_add(const MassW& W, float f0, float f1, float f2, float gm, float (&g)[3]) {
+    float h[20], p2[10];
+    mass_hidden1(W, f0, f1, f2, h);
+    mass_hidden2(W, h, p2);
+#pragma unroll
+    for (int i = 0; i < 10; ++i) p2[i] = gm * W.w[290 + i] * (p2[i] > 0.f ? 1.f : expf(p2[i]));
+    float a0 = 0.f, a1 = 0.f, a2 = 0.f;
+#pragma unroll
+    for (int j = 0; j < 20; ++j) {
+        float s = 0.f;
+#pragma unroll
+        for (int i = 0; i < 10; ++i) s = fmaf(W.w[80 + 20 * i + j], p2[i], s);
+        s *= h[j] > 0.f ? 1.f : h[j] + 1.f;
+        a0 = fmaf(W.w[3 * j], s, a0);
+        a1 = fmaf(W.w[3 * j + 1], s, a1);
+        a2 = fmaf(W.w[3 * j + 2], s, a2);
+    }
+    g[0] += a0;
+    g[1] += a1;
+    g[2] += a2;
+}
 
 // Compute warps synchronise among themselves on named barrier 1 (the
 // MMA-issuing warp never joins it); nbar_and also ANDs a predicate over them.
@@ -356,10 +431,10 @@ struct ZMap {
 // mbarriers of the forward
 enum : int { FB_A1 = 0, FB_A2 = 2, FB_D1 = 3, FB_D2 = 5, FB_DRAIN = 6, FB_COUNT = 7 };
 
-template <bool TWO_NET, bool BF>
+template <bool BF>
 __global__ void __launch_bounds__(NTW, 1)
     k_mlp_tc_fwd(const float* __restrict__ feat, const float4* __restrict__ img, ZMap zm, int ntiles, int nsplit,
-              float M_scale, float a, float* __restrict__ M_out, Saved sv, int* __restrict__ err, TcCtl ctl) {
+              float M_scale, float* __restrict__ M_out, Saved sv, int* __restrict__ err, TcCtl ctl) {
     using L = Lay<BF>;
     using F = LayF<BF>;
     extern __shared__ __align__(1024) unsigned char sm[];
@@ -626,15 +701,7 @@ __global__ void __launch_bounds__(NTW, 1)
             if (!in) return;
             const float yv = b3[0] + ((p[0] + p[1]) + (p[2] + p[3]));
             if (sv.y) sv.y[vox] = yv;
-            if (TWO_NET) {
-                const float pl = sigmoidf(a * yv);
-                float u0, u1, u2;
-                M_out[vox] = M_scale * pl *
-                             mass_net<false>(vec + VEC_MASS, feat[vox], feat[N3 + vox], feat[2 * N3 + vox], 0.f, u0,
-                                             u1, u2);
-            } else {
-                M_out[vox] = M_scale * softplusf(yv);
-            }
+            if (M_out) M_out[vox] = M_scale * softplusf(yv);  // NULL: k_mass_fwd forms the two-network head's M
         };
 
         int tile = blockIdx.x, prev = -1, last_it = 0;
@@ -698,8 +765,8 @@ struct LayB {
     static constexpr uint32_t S_GV = S_A4 + L::NP * SZ_A4;
     static constexpr int NTS = 27 * TX * TY * HZ;  // z-folded g_v, Ts[27][TX][TY][HZ]
     static constexpr uint32_t S_TAIL = S_GV + 4 * NTS;
-    // g_y [TM], centre-value gradients [3 slots][3][TM], 8 barriers + TMEM slot
-    static constexpr uint32_t SMEM = S_TAIL + 4 * TM + 4 * 9 * TM + 80;
+    // g_y [TM], 8 barriers + TMEM slot
+    static constexpr uint32_t SMEM = S_TAIL + 4 * TM + 80;
     static_assert(SMEM <= 232448, "shared memory budget");
     static_assert(S_B3 % 128 == 0 && S_B4 % 128 == 0 && S_A3 % 128 == 0 && S_A4 % 128 == 0 && S_GV % 16 == 0 &&
                       A3_BUF % 128 == 0 && S_TAIL % 16 == 0,
@@ -714,9 +781,8 @@ constexpr uint32_t COL_D3B = 0, COL_D4B = 128;
 
 template <bool TWO_NET, bool BF>
 __global__ void __launch_bounds__(NTW, 1)
-    k_mlp_tc_bwd(const float* __restrict__ feat, const float* __restrict__ gM, const float4* __restrict__ img,
-              TileMap tm, int ntiles, int nsplit, float M_scale, float a, float* __restrict__ gbox, Saved sv,
-              int* __restrict__ err, TcCtl ctl) {
+    k_mlp_tc_bwd(const float* __restrict__ gM, const float4* __restrict__ img, TileMap tm, int ntiles, int nsplit,
+              float M_scale, float a, float* __restrict__ gbox, Saved sv, int* __restrict__ err, TcCtl ctl) {
     using L = Lay<BF>;
     using B = LayB<BF>;
     extern __shared__ __align__(1024) unsigned char sm[];
@@ -724,8 +790,7 @@ __global__ void __launch_bounds__(NTW, 1)
     unsigned char* A4l = A4h + (L::NP - 1) * B::SZ_A4;
     float* gvs = reinterpret_cast<float*>(sm + B::S_GV);  // Ts[27][TX][TY][HZ]
     float* gys = reinterpret_cast<float*>(sm + B::S_TAIL);
-    float* gcen = gys + TM;  // [3 slots][3][TM]
-    uint64_t* bars = reinterpret_cast<uint64_t*>(gcen + 9 * TM);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(gys + TM);
     uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + BB_COUNT);
     const float* vec = reinterpret_cast<const float*>(sm + B::S_VEC);
     const float* w3 = vec + 96;
@@ -825,9 +890,9 @@ __global__ void __launch_bounds__(NTW, 1)
             y0 = ty * TY;
             z0 = tz * TZ;
         };
-        // saved forward state of a tile, loaded one tile ahead: g_M, y and the
-        // centre values of rows tid < TM; the masks of this thread's row and column block
-        float L_gm = 0.f, L_y = 0.f, L_f[3] = {0.f, 0.f, 0.f};
+        // saved forward state of a tile, loaded one tile ahead: g_M, y and the mass network's
+        // output of rows tid < TM; the masks of this thread's row and column block
+        float L_gm = 0.f, L_y = 0.f, L_mass = 0.f;
         uint32_t L_m1 = 0, L_m2 = 0;
         auto load_saved = [&](int tile) {
             if (tile >= ntiles) return;
@@ -839,9 +904,7 @@ __global__ void __launch_bounds__(NTW, 1)
                 const int64_t v = ((int64_t)gx * N + gy) * N + gz;
                 L_gm = in ? gM[v] : 0.f;
                 L_y = in ? sv.y[v] : 0.f;
-                if (TWO_NET)
-#pragma unroll
-                    for (int c = 0; c < 3; ++c) L_f[c] = in ? feat[c * N3 + v] : 0.f;
+                if (TWO_NET) L_mass = in ? sv.mass[v] : 0.f;
             }
             const int gx = x0 + (row >> 6), gy = y0 + ((row >> 4) & 3), gz = z0 + (row & 15);
             const bool in = gx < N && gy < N && gz < N;
@@ -850,8 +913,8 @@ __global__ void __launch_bounds__(NTW, 1)
             L_m2 = in ? sv.m2[cb * N3 + v] : 0u;
         };
         // g_y of the loaded tile, A3 = g_a2 = w3 g_y [a2 > 0] into A3 buffer b, arrive on
-        // its "A3 full"; the centre-value gradients (two-network head) into gcen slot `slot`
-        auto build_A3 = [&](int tile, int b, int slot) {
+        // its "A3 full"
+        auto build_A3 = [&](int tile, int b) {
             unsigned char* A3h = sm + B::S_A3 + (uint32_t)b * B::A3_BUF;
             unsigned char* A3l = A3h + (L::NP - 1) * B::SZ_A3;  // == A3h with one part
             int x0, y0, z0;
@@ -862,14 +925,9 @@ __global__ void __launch_bounds__(NTW, 1)
                 const bool in = gx < N && gy < N && gz < N;
                 const float g = in ? L_gm * M_scale : 0.f;
                 if (TWO_NET) {
-                    // M = M_scale p m: dM/dy = M_scale m a p (1 - p); dM/dm = M_scale p
+                    // M = M_scale p m: dM/dy = M_scale m a p (1 - p)
                     const float p = sigmoidf(a * L_y);
-                    float g0, g1, g2;
-                    const float m = mass_net<true>(vec + VEC_MASS, L_f[0], L_f[1], L_f[2], g * p, g0, g1, g2);
-                    gys[r] = g * m * a * p * (1.f - p);
-                    gcen[(slot * 3 + 0) * TM + r] = g0;
-                    gcen[(slot * 3 + 1) * TM + r] = g1;
-                    gcen[(slot * 3 + 2) * TM + r] = g2;
+                    gys[r] = g * L_mass * a * p * (1.f - p);
                 } else {
                     gys[r] = g * sigmoidf(L_y);
                 }
@@ -929,7 +987,7 @@ __global__ void __launch_bounds__(NTW, 1)
             box_mask |= msk << (9 * j);
         }
 
-        // g_v of a tile from D4 buffer b (gcen slot `slot`), folded over the z offset in
+        // g_v of a tile from D4 buffer b, folded over the z offset in
         // registers: a thread holds 24 columns = 8 whole (c, ox, oy) triples over oz
         // (k = 3 q + oz + 1), and the voxels z - 1, z + 1 of its row are the neighbouring
         // lanes of its 16-lane group, so T_q(hz) = g_v[q, oz=-1](hz) + g_v[q, 0](hz - 1) +
@@ -938,7 +996,7 @@ __global__ void __launch_bounds__(NTW, 1)
         // Ts[q][lx][ly][hz] (27 x 2 x 4 x 18; rows outside the mesh give 0). Then the box
         // sums: field c at box cell (hx, hy, hz) collects T of the triples (c, ox, oy) at
         // tile (lx, ly) = (hx - 1 - ox, hy - 1 - oy), in a fixed order.
-        auto epilogue4 = [&](int tile, int b, int slot) {
+        auto epilogue4 = [&](int tile, int b) {
             int x0, y0, z0;
             tile_origin(tile, x0, y0, z0);
             {
@@ -951,16 +1009,9 @@ __global__ void __launch_bounds__(NTW, 1)
                 for (int h = 0; h < 3; ++h) {
                     float av[8];
                     tmem_ld8(lane_base + COL_D4B + (uint32_t)b * 128 + 24 * cb + 8 * h, av);
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const int k = 24 * cb + 8 * h + j;
-                        float v = in ? av[j] : 0.f;
-                        if (TWO_NET && k < NI && k % 27 == 13 && in) v += gcen[(slot * 3 + k / 27) * TM + row];
-                        av[j] = v;
-                    }
                     // a load of 8 columns is not a whole number of triples: regroup
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) trip[(8 * h + j) / 3][(8 * h + j) % 3] = av[j];
+                    for (int j = 0; j < 8; ++j) trip[(8 * h + j) / 3][(8 * h + j) % 3] = in ? av[j] : 0.f;
                 }
 #pragma unroll
                 for (int t = 0; t < 8; ++t) {
@@ -994,14 +1045,14 @@ __global__ void __launch_bounds__(NTW, 1)
                             acc += gvs[box_base[j] + ((ox + 1) * 3 + (oy + 1)) * (TX * TY * HZ) - (ox * TY + oy) * HZ];
                 gbox[(int64_t)tile * NBOX + e] = acc;
             }
-            // the next writes of Ts and gcen come after the next tile's barriers
+            // the next writes of Ts come after the next tile's barriers
         };
 
         int tile = blockIdx.x, prev = -1, last_it = 0;
         uint32_t m1_cur = 0;
         load_saved(tile);
         if (tile < ntiles) {
-            build_A3(tile, 0, 0);
+            build_A3(tile, 0);
             m1_cur = L_m1;
             load_saved(tile + gridDim.x);
         }
@@ -1015,18 +1066,18 @@ __global__ void __launch_bounds__(NTW, 1)
             // (3) the next tile's A3 (its buffer's previous MMA3 and D3 reads are done)
             uint32_t m1_nxt = 0;
             if (nxt < ntiles) {
-                build_A3(nxt, b ^ 1, (it + 1) % 3);
+                build_A3(nxt, b ^ 1);
                 m1_nxt = L_m1;
                 load_saved(nxt + gridDim.x);
             }
             // (4) g_v and box sums of the previous tile while this tile's MMA4 runs
-            if (prev >= 0) epilogue4(prev, b ^ 1, (it + 2) % 3);
+            if (prev >= 0) epilogue4(prev, b ^ 1);
             m1_cur = m1_nxt;
             prev = tile;
         }
         if (ok && prev >= 0) {
             const int b = (last_it - 1) & 1;
-            if ((ok = wait_commit(BB_D4 + b, ph4, b))) epilogue4(prev, b, (last_it - 1) % 3);
+            if ((ok = wait_commit(BB_D4 + b, ph4, b))) epilogue4(prev, b);
         }
         if (!ok && tid == 0) atomicExch(err, 1);
     }
@@ -1125,8 +1176,20 @@ __device__ __forceinline__ int axis_boxes(int x, int N, int* t_out, int* b_out) 
     return n;
 }
 
-// g_field[c](cell) = sum over the tiles whose box holds the cell, in a fixed order.
+// What the two-network head adds to the input gradient: the mass network reads
+// the voxel's own fields, M = M_scale sigmoid(a y) m, so with g = gM M_scale
+// sigmoid(a y) the three fields' gradients grow by g dm/df_c.
+struct MassGrad {
+    MassW W;
+    const float *feat, *gM, *y;
+    float M_scale, a;
+};
+
+// g_field[c](cell) = sum over the tiles whose box holds the cell, in a fixed
+// order (+ the mass network's part, whose arithmetic hides behind the box loads).
+template <bool TWO_NET>
 __global__ void __launch_bounds__(256) k_stencil_tiles(const float* __restrict__ gbox, int N, int nty, int ntz,
+                                                       const __grid_constant__ MassGrad mg,
                                                        float* __restrict__ gfeat) {
     const int64_t N3 = (int64_t)N * N * N;
     const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1144,6 +1207,9 @@ __global__ void __launch_bounds__(256) k_stencil_tiles(const float* __restrict__
 #pragma unroll
                 for (int c = 0; c < 3; ++c) acc[c] += b[c * BOX];
             }
+    if (TWO_NET)
+        mass_grad_add(mg.W, mg.feat[v], mg.feat[N3 + v], mg.feat[2 * N3 + v],
+                      mg.gM[v] * mg.M_scale * sigmoidf(mg.a * mg.y[v]), acc);
 #pragma unroll
     for (int c = 0; c < 3; ++c) gfeat[c * N3 + v] = acc[c];
 }
@@ -1164,21 +1230,24 @@ std::vector<unsigned char> build_image(const float* W) {
     for (int h = 0; h < H2; ++h) vec[64 + h] = W[OFF_B2 + h];
     for (int h = 0; h < H2; ++h) vec[96 + h] = W[OFF_W3 + h];
     vec[128] = W[OFF_B3];
-    for (int i = 0; i < kMassWeights; ++i) vec[VEC_MASS + i] = W[OFF_B3 + 1 + i];  // zeros unless head == 1
     std::memcpy(&img[L::S_VEC], vec, SZ_VEC);
     return img;
 }
 
 template <bool BF>
 int set_smem_attrs(pmr_ctx* c) {
-    PMR_TRY(check_cuda(c, cudaFuncSetAttribute(k_mlp_tc_fwd<false, BF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)LayF<BF>::SMEM), "smem attr"));
-    PMR_TRY(check_cuda(c, cudaFuncSetAttribute(k_mlp_tc_fwd<true, BF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    PMR_TRY(check_cuda(c, cudaFuncSetAttribute(k_mlp_tc_fwd<BF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                (int)LayF<BF>::SMEM), "smem attr"));
     PMR_TRY(check_cuda(c, cudaFuncSetAttribute(k_mlp_tc_bwd<false, BF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                (int)LayB<BF>::SMEM), "smem attr"));
     return check_cuda(c, cudaFuncSetAttribute(k_mlp_tc_bwd<true, BF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)LayB<BF>::SMEM), "smem attr");
+}
+
+MassW mass_weights(const pmr_ctx* c) {
+    MassW W;
+    std::copy_n(c->W_host.begin() + OFF_B3 + 1, kMassWeights, W.w);
+    return W;
 }
 
 template <bool BWD, bool BF>
@@ -1187,7 +1256,7 @@ int launch_tc(pmr_ctx* c, const float* feat, const float* gM, float* M, int nspl
     TileMap m = tile_map(c, &ntiles);
     const float4* img = reinterpret_cast<const float4*>(BF ? c->tc_img_bf : c->tc_img);
     const float Ms = (float)c->cfg.M_scale;
-    const Saved sv{c->nn_y, c->nn_m1, c->nn_m2};  // written by the forward, read by the backward
+    const Saved sv{c->nn_y, c->nn_m1, c->nn_m2, c->nn_mass};  // written by the forward, read by the backward
     const TcCtl ctl{c->tc_stall ? kTestWaitLimit : kWaitLimit, c->tc_stall ? 0 : 1};
     if (!BWD) {
         // z-line tiles: N^2 lines of ceil(N / 128) segments
@@ -1200,21 +1269,21 @@ int launch_tc(pmr_ctx* c, const float* feat, const float* gM, float* M, int nspl
         const int nz_tiles = c->N * c->N * nzt;
         const int gz = std::min(nz_tiles, c->num_sms);
         const uint32_t sf = LayF<BF>::SMEM;
-        if (c->cfg.head == 1)
-            k_mlp_tc_fwd<true, BF><<<gz, NTW, sf, c->stream>>>(feat, img, zm, nz_tiles, nsplit, Ms, a, M, sv,
-                                                               c->tc_err, ctl);
-        else
-            k_mlp_tc_fwd<false, BF><<<gz, NTW, sf, c->stream>>>(feat, img, zm, nz_tiles, nsplit, Ms, a, M, sv,
-                                                                c->tc_err, ctl);
-        return check_launch(c, "mlp_tc_fwd");
+        k_mlp_tc_fwd<BF><<<gz, NTW, sf, c->stream>>>(feat, img, zm, nz_tiles, nsplit, Ms,
+                                                     c->cfg.head == 1 ? nullptr : M, sv, c->tc_err, ctl);
+        PMR_TRY(check_launch(c, "mlp_tc_fwd"));
+        if (c->cfg.head != 1) return PMR_OK;
+        k_mass_fwd<<<nblocks(c->N3, kMassT), kMassT, 0, c->stream>>>(mass_weights(c), feat, c->nn_y, c->N3, Ms, a,
+                                                                     c->nn_mass, M);
+        return check_launch(c, "mass_fwd");
     }
     const int grid = std::min(ntiles, c->num_sms);
     const uint32_t sb = LayB<BF>::SMEM;
     if (c->cfg.head == 1)
-        k_mlp_tc_bwd<true, BF><<<grid, NTW, sb, c->stream>>>(feat, gM, img, m, ntiles, nsplit, Ms, a, c->gbox, sv,
+        k_mlp_tc_bwd<true, BF><<<grid, NTW, sb, c->stream>>>(gM, img, m, ntiles, nsplit, Ms, a, c->gbox, sv,
                                                           c->tc_err, ctl);
     else
-        k_mlp_tc_bwd<false, BF><<<grid, NTW, sb, c->stream>>>(feat, gM, img, m, ntiles, nsplit, Ms, a, c->gbox, sv,
+        k_mlp_tc_bwd<false, BF><<<grid, NTW, sb, c->stream>>>(gM, img, m, ntiles, nsplit, Ms, a, c->gbox, sv,
                                                            c->tc_err, ctl);
     return check_launch(c, "mlp_tc_bwd");
 }
@@ -1248,10 +1317,17 @@ int mlp_tc_box_floats(int N) {
     return ((N + TX - 1) / TX) * ((N + TY - 1) / TY) * ((N + TZ - 1) / TZ) * 3 * HX * HY * HZ;
 }
 
-// input gradient of the three fields from the per-tile box sums of mlp_tc_backward_gv
-int stencil_tiles(pmr_ctx* c, float* gfeat) {
-    k_stencil_tiles<<<nblocks(c->N3, 256), 256, 0, c->stream>>>(c->gbox, c->N, (c->N + TY - 1) / TY,
-                                                                (c->N + TZ - 1) / TZ, gfeat);
+// input gradient of the three fields from the per-tile box sums of mlp_tc_backward_gv (and,
+// with the two-network head, the mass network's)
+int stencil_tiles(pmr_ctx* c, const float* feat, const float* gM, float a, float* gfeat) {
+    const int nty = (c->N + TY - 1) / TY, ntz = (c->N + TZ - 1) / TZ;
+    MassGrad mg{};
+    if (c->cfg.head == 1) {
+        mg = MassGrad{mass_weights(c), feat, gM, c->nn_y, (float)c->cfg.M_scale, a};
+        k_stencil_tiles<true><<<nblocks(c->N3, 256), 256, 0, c->stream>>>(c->gbox, c->N, nty, ntz, mg, gfeat);
+    } else {
+        k_stencil_tiles<false><<<nblocks(c->N3, 256), 256, 0, c->stream>>>(c->gbox, c->N, nty, ntz, mg, gfeat);
+    }
     return check_launch(c, "stencil_tiles");
 }
 
