@@ -219,7 +219,7 @@ int features_T(pmr_ctx* c, const float* gfeat, float* out) {
     Mul mul[3];
     for (int j = 0; j < 3; ++j) mul[j] = gauss(c, c->cfg.R_feat[j]);
     const float* ins[3] = {gfeat, gfeat + c->N3, gfeat + 2 * c->N3};
-    return conv_Nto1(c, ins, mul, 3, out);
+    return conv_Nto1(c, ins, nullptr, 1.f, 0.f, mul, 3, out);
 }
 
 int loss_and_grad_impl(pmr_ctx* c, const float2* s, const float* data, const pmr_anneal* an, double* host,
@@ -278,7 +278,7 @@ size_t pmr_workspace_bytes(const pmr_config* cfg) {
     size_t total = 0;
     for_each_buffer(*cfg, nullptr, [&](void**, size_t b) { total += (b + 255) / 256 * 256; });
     total += lbfgs_bytes(*cfg);
-    total += sizeof(float2) * (cfg->N + cfg->N / 2);  // twiddles
+    total += sizeof(float2) * cfg->N;  // twiddles
     return total;
 }
 
@@ -389,7 +389,7 @@ int pmr_linear_field(pmr_ctx* c, const float* white, double amplitude, void* s_k
     if (!white || !s_k) return fail(c, PMR_EINVAL, "NULL argument");
     Mul m{MUL_POWER, 0, (float)amplitude, 0.f, 0};
     const float* ins[1] = {white};
-    return real_to_k(c, ins, &m, 1, (float2*)s_k);
+    return real_to_k(c, ins, nullptr, 1.f, 0.f, &m, 1, (float2*)s_k, false);
 }
 
 int pm_forward(pmr_ctx* c, const void* s_k, float* delta_out) {

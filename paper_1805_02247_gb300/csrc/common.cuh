@@ -81,18 +81,7 @@ __device__ __forceinline__ float mass_net(const float* __restrict__ w, float f0,
 }
 #endif
 
-// Radix schedule of a 1D FFT of length n (Stockham autosort, radices 4/3/2),
-// with the per-stage divisors the butterflies need.
-struct Radix {
-    int n;
-    int nr;
-    int r[12];
-    FastDiv ns[12];   // Ns of stage s (product of the earlier radices)
-    FastDiv nrd[12];  // n / r[s]
-};
-
-Radix make_radix(int n);
-bool radix_ok(int n);
+bool radix_ok(int n);  // n = 2^a 3^b, n >= 2
 
 // Fourier-space multiplier applied inside the fused x-pass.
 enum MulType : int { MUL_ONE = 0, MUL_GAUSS = 1, MUL_ODD = 2, MUL_POWER = 3, MUL_HESS = 4 };
@@ -105,11 +94,11 @@ struct Mul {
     int i2;       // second component for MUL_HESS (k_j k_i2 / k^2)
 };
 
+struct FFTOps;  // launches of one mesh side's passes (fft_args.cuh)
 struct FFTPlan {
-    int N = 0, M = 0, P = 0;
-    Radix rN{}, rM{};
+    int N = 0;
+    const FFTOps* ops = nullptr;
     float2* twN = nullptr;  // exp(-2 pi i t / N), t < N (device)
-    float2* twM = nullptr;  // exp(-2 pi i t / M), t < M (device)
 };
 
 // Stored L-BFGS history on the device (float64), oldest first in a ring.
@@ -267,14 +256,19 @@ int fft_r2c(pmr_ctx* c, const float* in, float2* out);
 int fft_c2r(pmr_ctx* c, const float2* in, float* out, float2* work);
 // real in -> nout real outs, out_j = irfft(mul_j * rfft(in))
 int conv_1toN(pmr_ctx* c, const float* in, float* const* out, const Mul* mul, int nout);
+// out_i = irfft(mul * rfft(in_i)), i < n <= 3
+int conv_each(pmr_ctx* c, const float* const* in, float* const* out, const Mul& mul, int n);
+// The functions below with in2 take the inputs ca in_i + cb in2_i instead of in_i
+// (in2 may be NULL); with out2 they write s1 out_j and s2 out_j to the two outputs.
 // nin real ins -> real out = irfft(sum_i mul_i * rfft(in_i))
-int conv_Nto1(pmr_ctx* c, const float* const* in, const Mul* mul, int nin, float* out);
+int conv_Nto1(pmr_ctx* c, const float* const* in, const float* const* in2, float ca, float cb, const Mul* mul, int nin,
+              float* out);
 // k-space in (half array) -> nout real outs, out_j = irfft(mul_j * in)
-int k_to_real(pmr_ctx* c, const float2* in, float* const* out, const Mul* mul, int nout);
-// nin real ins -> k-space out = sum_i mul_i * rfft(in_i)
-int real_to_k(pmr_ctx* c, const float* const* in, const Mul* mul, int nin, float2* out);
-// out += sum_i mul_i rfft(in_i)
-int real_to_k_add(pmr_ctx* c, const float* const* in, const Mul* mul, int nin, float2* out);
+int k_to_real(pmr_ctx* c, const float2* in, float* const* out, const Mul* mul, int nout, float* const* out2 = nullptr,
+              float s1 = 1.f, float s2 = 1.f);
+// nin real ins -> k-space out = sum_i mul_i * rfft(in_i), added to out if add
+int real_to_k(pmr_ctx* c, const float* const* in, const float* const* in2, float ca, float cb, const Mul* mul, int nin,
+              float2* out, bool add);
 
 // PM kernels (pm.cu) ------------------------------------------------------------
 // positions are either explicit absolute positions (lattice == false) or

@@ -1,0 +1,63 @@
+// Arguments of the FFT passes and the launch table of one mesh side's plan.
+#pragma once
+
+#include "common.cuh"
+
+namespace pmr {
+
+// Element offsets of a half array: kz < M at x sx + y sy + kz, kz = M at n0 + x nx + y ny.
+struct Lay {
+    int sx, sy, n0, nx, ny;
+};
+// One side of a column pass: the transform axis has stride es (Nyquist plane:
+// nes), the other mesh axis stride os (nos).
+struct Side {
+    int os, es, n0, nos, nes;
+};
+
+struct XFused {
+    const float2* in[3];
+    float2* out[3];
+    int nin, nout;
+    int fwd;  // forward transform along x before the multiply
+    int inv;  // inverse transform along x after it
+    int acc;  // add the result to out instead of storing it
+    Mul mul[3];
+    const float* ptab;  // sqrt power table for MUL_POWER
+};
+
+// Up to three forward z transforms: in = a, or ca a + cb b where b is set.
+struct ZFwd {
+    const float* a[3];
+    const float* b[3];
+    float ca, cb;
+    float2* out[3];
+};
+
+// Up to three inverse z transforms: out = the transform x scale; with out2,
+// out = s1 times it and out2 = s2 times it.
+struct ZInv {
+    const float2* in[3];
+    float* out[3];
+    float* out2[3];
+    float s1, s2;
+};
+
+// x-pass variants: one input and one output (any number of such pairs, one
+// multiplier); one input and several outputs; several inputs and one output; the
+// ODD forms are for the three gradient components (multiplier o is MUL_ODD with
+// j = o, one scale and weighting), whose shared factor is applied once.
+enum XMode : int { X_1TO1 = 0, X_1TO3_ODD = 1, X_3TO1_ODD = 2, X_1TON = 3, X_NTO1 = 4 };
+
+// The launches of one mesh side's plan.
+struct FFTOps {
+    void (*z_r2c)(const ZFwd& p, int batch, const float2* tw, cudaStream_t s);
+    void (*z_c2r)(const ZInv& p, int batch, float scale, const float2* tw, cudaStream_t s);
+    void (*col)(const float2* in, const Side& si, float2* out, const Side& so, int64_t bs, int batch, bool inv,
+                const float2* tw, cudaStream_t s);
+    void (*x)(int mode, const XFused& p, const Side& si, const Side& so, int batch, const float2* tw, cudaStream_t s);
+    // calls set(kernel, dynamic shared-memory bytes) for every kernel of the plan
+    void (*each_kernel)(void (*set)(void* arg, const void* fn, size_t bytes), void* arg);
+};
+
+}  // namespace pmr

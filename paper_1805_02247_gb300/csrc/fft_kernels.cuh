@@ -1,0 +1,848 @@
+// Kernels of the 3D real FFTs on the N^3 mesh: three passes (z, y, x) of register four-step
+// transforms, with the Fourier-space multipliers of the method (PM Green's
+// function and gradient, Gaussian smoothing, Zel'dovich displacement, linear
+// power) fused into the x-pass, where every element holds its full (kx, ky, kz)
+// value.
+//
+// Forward r2c = z-pass (real rows -> half complex), y-pass, x-pass.
+// Inverse c2r = x-pass, y-pass, z-pass (half complex -> real rows, 1/N^3).
+// Each pass reads and writes the array once. Every mesh side a context takes
+// (N = 2^a 3^b, 8..512) has a compile-time plan: a 1D transform of length
+// n = N1 N2 runs as two rounds of DFTs held in registers with one transpose
+// through shared memory in between.
+//
+// Layouts of the half array. The caller's (ABI) layout is [x][y][kz <= M],
+// M = N/2. Its rows are M + 1 values long, so the 128-byte pieces a pass's tile
+// takes of them straddle lines (five 32-byte sectors instead of four), and the
+// last tile of each row holds one column. The library's own arrays keep the
+// Nyquist plane apart: [x][y][kz < M], then [x][y] for kz = M. The z passes use
+// that one; the y and x passes take either on either side (Lay).
+#pragma once
+
+#include <type_traits>
+#include <utility>
+
+#include "fft_args.cuh"
+
+namespace pmr {
+
+namespace {
+
+__device__ __forceinline__ float2 cmul(float2 a, float2 b) {
+    return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+}
+__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
+__device__ __forceinline__ float2 cscale(float2 a, float s) { return make_float2(a.x * s, a.y * s); }
+
+// ----------------------------------------------------------------------------- small DFTs
+
+// cos(2 pi u / r) or sin(2 pi u / r) at compile time: the angle is folded to
+// m pi/2 +- a with a in [0, pi/4], then the Taylor series in double.
+constexpr double taylor_cs(double a, bool sine) {
+    double term = sine ? a : 1.0, sum = term;
+    for (int k = sine ? 2 : 1; k < 24; k += 2) {
+        term *= -a * a / (double)(k * (k + 1));
+        sum += term;
+    }
+    return sum;
+}
+constexpr double root_cs(int u, int r, bool sine) {
+    const int oct = 8 * u / r % 8, rem = 8 * u - r * (8 * u / r);
+    const bool odd = oct % 2 == 1;
+    const double a = (double)(odd ? r - rem : rem) / (double)r * 0.78539816339744830962;
+    const int m = (odd ? oct + 1 : oct) / 2 % 4;
+    const double c = taylor_cs(a, false), s = odd ? -taylor_cs(a, true) : taylor_cs(a, true);
+    const double cs[4] = {c, -s, -c, s}, sn[4] = {s, c, -s, -c};
+    return sine ? sn[m] : cs[m];
+}
+
+// a times exp(-2 pi i U / R) (INV: its conjugate); the root is an immediate of
+// the multiplications, and quarter turns take none
+template <int U, int R, bool INV>
+__device__ __forceinline__ float2 root_mul(float2 a) {
+    constexpr int u = U % R;
+    if constexpr (u == 0) {
+        return a;
+    } else if constexpr (2 * u == R) {
+        return make_float2(-a.x, -a.y);
+    } else if constexpr (4 * u == R || 4 * u == 3 * R) {
+        constexpr bool plus_i = (4 * u == R) == INV;
+        return plus_i ? make_float2(-a.y, a.x) : make_float2(a.y, -a.x);
+    } else {
+        constexpr float c = (float)root_cs(u, R, false), s = (float)root_cs(u, R, true);
+        return cmul(a, make_float2(c, INV ? s : -s));
+    }
+}
+
+template <class F, int... I>
+__device__ __forceinline__ void static_for_impl(F f, std::integer_sequence<int, I...>) {
+    (f(std::integral_constant<int, I>{}), ...);
+}
+template <int N, class F>
+__device__ __forceinline__ void static_for(F f) {
+    static_for_impl(f, std::make_integer_sequence<int, N>{});
+}
+
+// R-point DFT in registers, R = 2^a 3^b; INV uses exp(+2 pi i / R). R > 4 by
+// decimation: X[k + s q] = sum_j W_R^(jk) S_j[k] W_r^(jq), S_j the s-point DFT of x[r m + j].
+template <int R, bool INV>
+__device__ __forceinline__ void dft_reg(float2* v) {
+    if constexpr (R == 2) {
+        const float2 a = v[0], b = v[1];
+        v[0] = cadd(a, b);
+        v[1] = csub(a, b);
+    } else if constexpr (R == 4) {
+        const float2 t0 = cadd(v[0], v[2]), t1 = csub(v[0], v[2]);
+        const float2 t2 = cadd(v[1], v[3]), d = csub(v[1], v[3]);
+        // forward: -i * d, inverse: +i * d
+        const float2 t3 = INV ? make_float2(-d.y, d.x) : make_float2(d.y, -d.x);
+        v[0] = cadd(t0, t2);
+        v[2] = csub(t0, t2);
+        v[1] = cadd(t1, t3);
+        v[3] = csub(t1, t3);
+    } else if constexpr (R == 3) {
+        const float h = 0.86602540378443864676f;  // sqrt(3)/2
+        const float2 a = v[0], s = cadd(v[1], v[2]), d = csub(v[1], v[2]);
+        const float2 m = make_float2(a.x - 0.5f * s.x, a.y - 0.5f * s.y);
+        // +-i h d
+        const float2 r = INV ? make_float2(-h * d.y, h * d.x) : make_float2(h * d.y, -h * d.x);
+        v[0] = cadd(a, s);
+        v[1] = cadd(m, r);
+        v[2] = csub(m, r);
+    } else if constexpr (R > 4) {
+        constexpr int r = (R % 4 == 0) ? 4 : (R % 2 == 0) ? 2 : 3;
+        constexpr int s = R / r;
+        float2 sub[r][s];
+#pragma unroll
+        for (int j = 0; j < r; ++j)
+#pragma unroll
+            for (int m = 0; m < s; ++m) sub[j][m] = v[r * m + j];
+#pragma unroll
+        for (int j = 0; j < r; ++j) dft_reg<s, INV>(sub[j]);
+        static_for<s>([&](auto k) {
+            float2 t[r];
+            static_for<r>([&](auto j) { t[j] = root_mul<j * k, R, INV>(sub[j][k]); });
+            dft_reg<r, INV>(t);
+#pragma unroll
+            for (int q = 0; q < r; ++q) v[k + s * q] = t[q];
+        });
+    }
+}
+
+// ----------------------------------------------------------------------------- multipliers
+
+__device__ __forceinline__ float2 apply_mul(const Mul& m, float2 v, int nx, int ny, int kz, int N,
+                                            const float* __restrict__ ptab) {
+    const float twopi_n = 6.28318530717958647692f / (float)N;
+    float f = m.scale;
+    if (m.weighted) f *= (kz == 0 || 2 * kz == N) ? 1.0f : 2.0f;
+    if (m.type == MUL_ONE) return cscale(v, f);
+    const int n2 = nx * nx + ny * ny + kz * kz;
+    if (m.type == MUL_POWER) return cscale(v, f * ptab[n2]);
+    const float kx = twopi_n * nx, ky = twopi_n * ny, kzf = twopi_n * kz;
+    const float k2 = kx * kx + ky * ky + kzf * kzf;
+    if (m.type == MUL_GAUSS) return cscale(v, f * expf(-0.5f * k2 * m.R2));
+    if (m.type == MUL_HESS) {
+        // k_j k_i2 / k^2, zero at k = 0; for j != i2 also zero where either
+        // component is the Nyquist frequency (an odd factor there)
+        const int na = (m.j == 0) ? nx : (m.j == 1) ? ny : kz;
+        const int nb = (m.i2 == 0) ? nx : (m.i2 == 1) ? ny : kz;
+        if (n2 == 0 || (m.j != m.i2 && (2 * abs(na) == N || 2 * abs(nb) == N))) return make_float2(0.f, 0.f);
+        return cscale(v, f * (twopi_n * na) * (twopi_n * nb) / k2);
+    }
+    // MUL_ODD: i k_j / k^2, zero at k = 0 and on the Nyquist plane of component j
+    const int nj = (m.j == 0) ? nx : (m.j == 1) ? ny : kz;
+    if (n2 == 0 || 2 * abs(nj) == N) return make_float2(0.f, 0.f);
+    const float kj = twopi_n * nj;
+    const float a = f * kj / k2;
+    return make_float2(-a * v.y, a * v.x);
+}
+
+// the parts of MUL_ODD: f / k^2 (0 at k = 0), and k_j (0 on the Nyquist plane of j)
+__device__ __forceinline__ float odd_g(const Mul& m, int nx, int ny, int kz, int N) {
+    const int n2 = nx * nx + ny * ny + kz * kz;
+    if (n2 == 0) return 0.f;
+    const float twopi_n = 6.28318530717958647692f / (float)N;
+    float f = m.scale;
+    if (m.weighted) f *= (kz == 0 || 2 * kz == N) ? 1.0f : 2.0f;
+    const float kx = twopi_n * nx, ky = twopi_n * ny, kzf = twopi_n * kz;
+    return f / (kx * kx + ky * ky + kzf * kzf);
+}
+__device__ __forceinline__ float odd_k(int j, int nx, int ny, int kz, int N) {
+    const int nj = (j == 0) ? nx : (j == 1) ? ny : kz;
+    return 2 * abs(nj) == N ? 0.f : (6.28318530717958647692f / (float)N) * nj;
+}
+
+// ----------------------------------------------------------------------------- column passes
+//
+// A block takes RC adjacent columns (one 128-byte line per row; 64 bytes where
+// 16 columns would leave one block per SM) and each 1D transform runs as the
+// four-step decomposition:
+//   forward order:  x[N2 n1 + n2]  --DFT_N1 over n1, x W^(n2 k1), DFT_N2 over n2-->  X[k1 + N1 k2]
+//   inverse order:  X[k1 + N1 k2]  --DFT_N2 over k2, x W^(n2 k1), DFT_N1 over k1-->  x[n2 + N2 n1]
+// Either order computes a DFT of either sign. A thread owns one column and a
+// set of n2 (rows N2 n1 + n2) or of k1 (rows k1 + N1 k2), so every global
+// access of a warp is whole rows of the tile and no index needs a division.
+// Blocks with blockIdx.y >= N take the Nyquist plane, RC lines of it each.
+
+constexpr int cgcd(int a, int b) { return b == 0 ? a : cgcd(b, a % b); }
+
+template <int N1_, int N2_, int RC_ = 16>
+struct Reg {
+    static constexpr int N1 = N1_, N2 = N2_, N = N1 * N2;
+    static constexpr int G = cgcd(N1, N2);       // threads per column
+    static constexpr int A1 = N2 / G;            // n2 values per thread
+    static constexpr int A2 = N1 / G;            // k1 values per thread
+    static_assert(N1 % G == 0 && N2 % G == 0, "factors must divide");
+    static constexpr int E = N / G;              // complex values per thread
+    static constexpr int RC = RC_;               // columns per block
+    static constexpr int T = RC * G;             // block size
+    // transpose buffer S[k1][n2][c]; with 8 columns a padding column set keeps
+    // neighbouring k1 on alternating halves of the banks
+    static constexpr int SP = RC == 8 ? N2 + 1 : N2;
+    static constexpr int S_ELEMS = N1 * SP * RC;
+    // twiddles + transpose buffer; + kept k-space tile (several outputs)
+    static constexpr size_t smem_col() { return sizeof(float2) * (size_t)(N + S_ELEMS); }
+    static constexpr size_t smem_kept() { return sizeof(float2) * (size_t)(N + S_ELEMS + N * RC); }
+    // several inputs: the running sum is in registers, or in shared memory where it would spill
+    static constexpr bool SUM_SMEM = E > 24;
+    static constexpr size_t smem_x(int mode) {
+        const bool many_out = mode == X_1TO3_ODD || mode == X_1TON, many_in = mode == X_3TO1_ODD || mode == X_NTO1;
+        return many_out || (many_in && SUM_SMEM) ? smem_kept() : smem_col();
+    }
+    // resident blocks of the fused x-pass: as many as `regs` registers a thread and
+    // the shared memory allow (at N = 256: 80 registers and 3 blocks for one input,
+    // 128 and 2 for several, which spill at 80)
+    static constexpr int xb(int mode) {
+        const bool sum_regs = (mode == X_3TO1_ODD || mode == X_NTO1) && !SUM_SMEM;
+        const int regs = sum_regs ? (E <= 16 ? 128 : 240) : (E <= 16 ? 80 : E <= 24 ? 112 : 240);
+        const int Tr = (T + 127) / 128 * 128;  // registers are allocated to four warps at a time
+        const int r = 65536 / (Tr * regs), s = (int)(232448 / smem_x(mode));
+        const int b = r < s ? r : s;
+        return b < 1 ? 1 : b > 16 ? 16 : b;
+    }
+};
+
+template <class RG>
+__device__ __forceinline__ int sidx(int k1, int n2, int c) {
+    return (k1 * RG::SP + n2) * RG::RC + c;
+}
+
+__device__ __forceinline__ void load_twiddles(float2* s_tw, const float2* g_tw, int n) {
+    for (int t = threadIdx.x; t < n; t += blockDim.x) s_tw[t] = g_tw[t];
+}
+
+// x[N2 n1 + n2] (thread owns n2 = g + G a) -> X[k1 + N1 k2] (thread owns k1 = g + G a)
+template <class RG, bool INV>
+__device__ __forceinline__ void four_step_fwd(float2 (&v1)[RG::A1][RG::N1], float2 (&v2)[RG::A2][RG::N2], float2* S,
+                                              const float2* tw, int c, int g) {
+    constexpr int N1 = RG::N1, N2 = RG::N2, G = RG::G;
+#pragma unroll
+    for (int a = 0; a < RG::A1; ++a) {
+        const int n2 = g + G * a;
+        dft_reg<N1, INV>(v1[a]);
+#pragma unroll
+        for (int k1 = 0; k1 < N1; ++k1) {
+            float2 v = v1[a][k1];
+            if (k1 > 0) {
+                float2 w = tw[n2 * k1];
+                if (INV) w.y = -w.y;
+                v = cmul(v, w);
+            }
+            S[sidx<RG>(k1, n2, c)] = v;
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int a = 0; a < RG::A2; ++a) {
+        const int k1 = g + G * a;
+#pragma unroll
+        for (int n2 = 0; n2 < N2; ++n2) v2[a][n2] = S[sidx<RG>(k1, n2, c)];
+        dft_reg<N2, INV>(v2[a]);
+    }
+}
+
+// X[k1 + N1 k2] (thread owns k1) -> x[n2 + N2 n1] (thread owns n2)
+template <class RG, bool INV>
+__device__ __forceinline__ void four_step_inv(float2 (&v2)[RG::A2][RG::N2], float2 (&v1)[RG::A1][RG::N1], float2* S,
+                                              const float2* tw, int c, int g) {
+    constexpr int N1 = RG::N1, N2 = RG::N2, G = RG::G;
+#pragma unroll
+    for (int a = 0; a < RG::A2; ++a) {
+        const int k1 = g + G * a;
+        dft_reg<N2, INV>(v2[a]);
+#pragma unroll
+        for (int n2 = 0; n2 < N2; ++n2) {
+            float2 v = v2[a][n2];
+            if (n2 > 0 && k1 > 0) {
+                float2 w = tw[n2 * k1];
+                if (INV) w.y = -w.y;
+                v = cmul(v, w);
+            }
+            S[sidx<RG>(k1, n2, c)] = v;
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int a = 0; a < RG::A1; ++a) {
+        const int n2 = g + G * a;
+#pragma unroll
+        for (int k1 = 0; k1 < N1; ++k1) v1[a][k1] = S[sidx<RG>(k1, n2, c)];
+        dft_reg<N1, INV>(v1[a]);
+    }
+}
+
+// rows N2 n1 + n2 of the thread's n2 set
+template <class RG>
+__device__ __forceinline__ void load_n2(float2 (&v1)[RG::A1][RG::N1], const float2* in, int es, bool ok, int g) {
+#pragma unroll
+    for (int a = 0; a < RG::A1; ++a)
+#pragma unroll
+        for (int n1 = 0; n1 < RG::N1; ++n1)
+            v1[a][n1] = ok ? in[(RG::N2 * n1 + g + RG::G * a) * es] : make_float2(0.f, 0.f);
+}
+
+// rows k1 + N1 k2 of the thread's k1 set
+template <class RG>
+__device__ __forceinline__ void load_k1(float2 (&v2)[RG::A2][RG::N2], const float2* in, int es, bool ok, int g) {
+#pragma unroll
+    for (int a = 0; a < RG::A2; ++a)
+#pragma unroll
+        for (int k2 = 0; k2 < RG::N2; ++k2)
+            v2[a][k2] = ok ? in[(g + RG::G * a + RG::N1 * k2) * es] : make_float2(0.f, 0.f);
+}
+
+__device__ __forceinline__ void put(float2* d, float2 v, bool acc) { *d = acc ? cadd(*d, v) : v; }
+
+// The thread's column: offsets of its element 0 on both sides, their strides,
+// its kz and other mesh coordinate.
+struct Column {
+    int in, ies, out, oes, kz, outer;
+    bool ok;
+};
+template <class RG>
+__device__ __forceinline__ Column column(const Side& si, const Side& so, int c) {
+    constexpr int M = RG::N / 2;
+    Column q;
+    if ((int)blockIdx.y < RG::N) {
+        q.outer = blockIdx.y;
+        q.kz = blockIdx.x * RG::RC + c;
+        q.ok = q.kz < M;
+        q.in = q.outer * si.os + q.kz;
+        q.out = q.outer * so.os + q.kz;
+        q.ies = si.es;
+        q.oes = so.es;
+    } else {
+        q.outer = (((int)blockIdx.y - RG::N) * gridDim.x + blockIdx.x) * RG::RC + c;
+        q.kz = M;
+        q.ok = q.outer < RG::N;
+        q.in = si.n0 + q.outer * si.nos;
+        q.out = so.n0 + q.outer * so.nos;
+        q.ies = si.nes;
+        q.oes = so.nes;
+    }
+    return q;
+}
+template <class RG>
+dim3 col_grid(int batch) {
+    const int nct = (RG::N / 2 + RG::RC - 1) / RG::RC, nyq = (RG::N + RG::RC - 1) / RG::RC;
+    return dim3(nct, RG::N + (nyq + nct - 1) / nct, batch);
+}
+
+// Plain y- or x-pass (no multiplier); in-place safe (a block's tile is read before
+// any of it is written, and tiles are disjoint). blockIdx.z: arrays, bs apart.
+template <class RG, bool INV>
+__global__ void __launch_bounds__(RG::T) k_col_reg(const float2* in, float2* out, int64_t bs, Side si, Side so,
+                                                     const float2* __restrict__ tw) {
+    extern __shared__ float2 sm[];
+    float2* s_tw = sm;
+    float2* S = s_tw + RG::N;
+    load_twiddles(s_tw, tw, RG::N);
+    const int c = threadIdx.x % RG::RC, g = threadIdx.x / RG::RC;
+    const Column q = column<RG>(si, so, c);
+    in += blockIdx.z * bs + q.in;
+    out += blockIdx.z * bs + q.out;
+    float2 v1[RG::A1][RG::N1], v2[RG::A2][RG::N2];
+    load_n2<RG>(v1, in, q.ies, q.ok, g);
+    __syncthreads();  // twiddles
+    four_step_fwd<RG, INV>(v1, v2, S, s_tw, c, g);
+    if (q.ok)
+#pragma unroll
+        for (int a = 0; a < RG::A2; ++a)
+#pragma unroll
+            for (int k2 = 0; k2 < RG::N2; ++k2) out[(g + RG::G * a + RG::N1 * k2) * q.oes] = v2[a][k2];
+}
+
+// x-pass with multipliers. Tile: outer index = ky row, columns = kz, transform
+// axis = x. out_j = [inv] mul_j * [fwd] in_0, or out_0 = [inv] sum_i mul_i * [fwd] in_i.
+// Several outputs keep the k-space tile in shared memory between them.
+template <class RG, int MODE>
+__global__ void __launch_bounds__(RG::T, RG::xb(MODE)) k_x_reg(const __grid_constant__ XFused p, Side si, Side so,
+                                                               const float2* __restrict__ tw) {
+    extern __shared__ float2 sm[];
+    constexpr int N = RG::N;
+    float2* s_tw = sm;
+    float2* S = s_tw + N;
+    load_twiddles(s_tw, tw, N);
+    const int c = threadIdx.x % RG::RC, g = threadIdx.x / RG::RC;
+    const Column q = column<RG>(si, so, c);
+    const bool ok = q.ok;
+    const int kz = q.kz;
+    const int ny = (2 * q.outer <= N) ? q.outer : q.outer - N;
+    __syncthreads();  // twiddles
+
+    float2* Kb = S + RG::S_ELEMS;  // kept k-space tile: value e of thread t at Kb[e * T + t]
+    float2 v1[RG::A1][RG::N1];
+    auto to_k = [&](const float2* src, float2 (&dst)[RG::A2][RG::N2]) {
+        if (p.fwd) {
+            load_n2<RG>(v1, src + q.in, q.ies, ok, g);
+            four_step_fwd<RG, false>(v1, dst, S, s_tw, c, g);
+            __syncthreads();  // S free again
+        } else {
+            load_k1<RG>(dst, src + q.in, q.ies, ok, g);
+        }
+    };
+    auto nx_of = [&](int a, int k2) {
+        const int mx = g + RG::G * a + RG::N1 * k2;
+        return (2 * mx <= N) ? mx : mx - N;
+    };
+    auto mul_into = [&](const Mul& m, const float2 (&src)[RG::A2][RG::N2], float2 (&dst)[RG::A2][RG::N2], bool add) {
+#pragma unroll
+        for (int a = 0; a < RG::A2; ++a)
+#pragma unroll
+            for (int k2 = 0; k2 < RG::N2; ++k2) {
+                // columns past the mesh stay zero and never index the power table
+                const float2 v =
+                    ok ? apply_mul(m, src[a][k2], nx_of(a, k2), ny, kz, N, p.ptab) : make_float2(0.f, 0.f);
+                dst[a][k2] = add ? cadd(dst[a][k2], v) : v;
+            }
+    };
+    // R (inverse transformed if p.inv) handed element by element to st(offset, value)
+    auto finish = [&](float2 (&R)[RG::A2][RG::N2], auto st) {
+        if (p.inv) {
+            four_step_inv<RG, true>(R, v1, S, s_tw, c, g);
+            if (ok)
+#pragma unroll
+                for (int a = 0; a < RG::A1; ++a)
+#pragma unroll
+                    for (int n1 = 0; n1 < RG::N1; ++n1)
+                        st(q.out + (g + RG::G * a + RG::N2 * n1) * q.oes, v1[a][n1]);
+        } else if (ok) {
+#pragma unroll
+            for (int a = 0; a < RG::A2; ++a)
+#pragma unroll
+                for (int k2 = 0; k2 < RG::N2; ++k2) st(q.out + (g + RG::G * a + RG::N1 * k2) * q.oes, R[a][k2]);
+        }
+    };
+    auto emit = [&](float2 (&R)[RG::A2][RG::N2], float2* dst) {
+        finish(R, [&](int o, float2 v) { put(dst + o, v, p.acc); });
+    };
+    float2 X[RG::A2][RG::N2];
+    float2* Kt = Kb + threadIdx.x;
+    if constexpr (MODE == X_1TO1) {
+        to_k(p.in[blockIdx.z], X);
+        mul_into(p.mul[0], X, X, false);
+        emit(X, p.out[blockIdx.z]);
+    } else if constexpr (MODE == X_1TO3_ODD) {
+        // kept tile: X f/k^2; output o is i k_o times it
+        to_k(p.in[0], X);
+#pragma unroll
+        for (int a = 0; a < RG::A2; ++a)
+#pragma unroll
+            for (int k2 = 0; k2 < RG::N2; ++k2) {
+                const float2 v = cscale(X[a][k2], ok ? odd_g(p.mul[0], nx_of(a, k2), ny, kz, N) : 0.f);
+                Kt[(a * RG::N2 + k2) * RG::T] = v;
+                // x component: its k_x varies along the transform axis
+                const float kj = odd_k(0, nx_of(a, k2), ny, kz, N);
+                X[a][k2] = make_float2(-kj * v.y, kj * v.x);
+            }
+        emit(X, p.out[0]);
+        // y and z components: k_y, k_z are constant along it, so both are i k_y and
+        // i k_z times one inverse transform of the kept tile
+#pragma unroll
+        for (int a = 0; a < RG::A2; ++a)
+#pragma unroll
+            for (int k2 = 0; k2 < RG::N2; ++k2) X[a][k2] = Kt[(a * RG::N2 + k2) * RG::T];
+        if (p.inv) __syncthreads();  // S free again
+        const float s1 = odd_k(1, 0, ny, kz, N), s2 = odd_k(2, 0, ny, kz, N);
+        finish(X, [&](int o, float2 v) {
+            p.out[1][o] = make_float2(-s1 * v.y, s1 * v.x);
+            p.out[2][o] = make_float2(-s2 * v.y, s2 * v.x);
+        });
+    } else if constexpr (MODE == X_1TON) {
+        to_k(p.in[0], X);
+#pragma unroll
+        for (int a = 0; a < RG::A2; ++a)
+#pragma unroll
+            for (int k2 = 0; k2 < RG::N2; ++k2) Kt[(a * RG::N2 + k2) * RG::T] = X[a][k2];
+#pragma unroll 1
+        for (int o = 0; o < p.nout; ++o) {
+            if (p.inv && o > 0) __syncthreads();  // S free again
+#pragma unroll
+            for (int a = 0; a < RG::A2; ++a)
+#pragma unroll
+                for (int k2 = 0; k2 < RG::N2; ++k2) X[a][k2] = Kt[(a * RG::N2 + k2) * RG::T];
+            mul_into(p.mul[o], X, X, false);
+            emit(X, p.out[o]);
+        }
+    } else {
+        // X_3TO1_ODD: sum_i k_i X_i, then times i f/k^2 once
+        float2 acc[RG::SUM_SMEM ? 1 : RG::A2][RG::SUM_SMEM ? 1 : RG::N2];
+#pragma unroll 1
+        for (int i = 0; i < p.nin; ++i) {
+            to_k(p.in[i], X);
+#pragma unroll
+            for (int a = 0; a < RG::A2; ++a)
+#pragma unroll
+                for (int k2 = 0; k2 < RG::N2; ++k2) {
+                    float2 v;
+                    if constexpr (MODE == X_3TO1_ODD)
+                        v = cscale(X[a][k2], odd_k(i, nx_of(a, k2), ny, kz, N));
+                    else  // columns past the mesh stay zero and never index the power table
+                        v = ok ? apply_mul(p.mul[i], X[a][k2], nx_of(a, k2), ny, kz, N, p.ptab) : make_float2(0.f, 0.f);
+                    if constexpr (RG::SUM_SMEM) {
+                        float2& s = Kt[(a * RG::N2 + k2) * RG::T];
+                        s = i > 0 ? cadd(s, v) : v;
+                    } else {
+                        acc[a][k2] = i > 0 ? cadd(acc[a][k2], v) : v;
+                    }
+                }
+        }
+#pragma unroll
+        for (int a = 0; a < RG::A2; ++a)
+#pragma unroll
+            for (int k2 = 0; k2 < RG::N2; ++k2) {
+                float2 v;
+                if constexpr (RG::SUM_SMEM)
+                    v = Kt[(a * RG::N2 + k2) * RG::T];
+                else
+                    v = acc[a][k2];
+                if constexpr (MODE == X_3TO1_ODD) {
+                    const float gk = ok ? odd_g(p.mul[0], nx_of(a, k2), ny, kz, N) : 0.f;
+                    v = make_float2(-gk * v.y, gk * v.x);
+                }
+                X[a][k2] = v;
+            }
+        emit(X, p.out[0]);
+    }
+}
+
+// ----------------------------------------------------------------------------- z passes
+//
+// Rows of N reals are M = N/2 complex points z_m = x_2m + i x_2m+1. A block
+// stages R rows in shared memory with coalesced loads and runs the M-point
+// transform of each row as the four-step order above, G threads a row, all of
+// one warp, so that warp barriers order the steps and the row's transpose uses
+// its own staging memory. The real-to-complex split is done on the registers:
+// the forward pass needs Z_k and Z_(M-k), which sit in threads g and G - g of
+// the row (two shuffles an element), and the inverse pass forms each z_k from
+// the staged X_k and X_(M-k) as it loads it.
+
+template <class RG>
+struct ZReg {
+    static constexpr int M = RG::N, N = 2 * M, G = RG::G;
+    static constexpr int T = 128;
+    static constexpr int RW = 32 / G;          // rows per warp (lanes past RW G repeat lane 0's work, storing nothing)
+    static constexpr int R = T / 32 * RW;      // rows per block
+    // Row pitch of the staging buffer, which also holds the row's transpose: wide
+    // enough for both, and = 8 mod 16 float2 so the rows of one warp fall on
+    // alternating halves of the banks.
+    static constexpr int NEED = (M + 9) > RG::N1 * (RG::N2 + 1) ? (M + 9) : RG::N1 * (RG::N2 + 1);
+    static constexpr int PITCH = (NEED + 7) / 16 * 16 + 8;
+    // split table W_N^k (k <= M, padded to 16 bytes), four-step table [k1][n2], rows
+    static constexpr int SPLIT = (M + 2) / 2 * 2;
+    static constexpr size_t smem() { return sizeof(float2) * (size_t)(SPLIT + (M + 1) / 2 * 2 + R * PITCH); }
+    static_assert(G <= 32, "a row's threads lie in one warp");
+};
+
+// The two twiddle tables of a z pass. The four-step's is laid out as it is read,
+// W_M^(n2 k1) at [k1][n2], so the threads of a row take consecutive entries (read
+// as W_N^(2 n2 k1) from one table, even k1 met up to eight-way bank conflicts).
+template <class Z, class RG>
+__device__ __forceinline__ void load_z_tables(float2* split, float2* four, const float2* __restrict__ twN) {
+    for (int t = threadIdx.x; t <= Z::M; t += Z::T) split[t] = twN[t];
+    for (int t = threadIdx.x; t < Z::M; t += Z::T) four[t] = twN[2 * (t / RG::N2) * (t % RG::N2)];
+}
+
+// rows x M values, contiguous at src, into the staging rows A (pitch PITCH); every
+// load of a thread is in flight before its first shared-memory store. Two values a
+// load where the source is 16-byte aligned and M even. src2: ca src + cb src2 instead.
+template <class Z>
+__device__ __forceinline__ void stage_rows(float2* A, const float2* __restrict__ src, int rows,
+                                           const float2* __restrict__ src2, float ca, float cb) {
+    constexpr int M = Z::M;
+    const int tid = threadIdx.x;
+    if constexpr (M % 2 == 0) {
+        if ((((uintptr_t)src | (uintptr_t)src2) & 15) == 0) {
+            constexpr int V = M / 2, LD = (Z::R * V + Z::T - 1) / Z::T;
+            const float4* s4 = reinterpret_cast<const float4*>(src);
+            float4 v[LD];
+#pragma unroll
+            for (int q = 0; q < LD; ++q) {
+                const int t = tid + q * Z::T;
+                v[q] = t < rows * V ? s4[t] : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+            if (src2) {
+                const float4* s42 = reinterpret_cast<const float4*>(src2);
+#pragma unroll
+                for (int q = 0; q < LD; ++q) {
+                    const int t = tid + q * Z::T;
+                    const float4 w = t < rows * V ? s42[t] : make_float4(0.f, 0.f, 0.f, 0.f);
+                    v[q] = make_float4(ca * v[q].x + cb * w.x, ca * v[q].y + cb * w.y, ca * v[q].z + cb * w.z,
+                                       ca * v[q].w + cb * w.w);
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < LD; ++q) {
+                const int t = tid + q * Z::T, r = t / V, m = t - r * V;
+                if (t < Z::R * V) *reinterpret_cast<float4*>(A + r * Z::PITCH + 2 * m) = v[q];
+            }
+            return;
+        }
+    }
+    constexpr int LD = (Z::R * M + Z::T - 1) / Z::T;
+    float2 v[LD];
+#pragma unroll
+    for (int q = 0; q < LD; ++q) {
+        const int t = tid + q * Z::T;
+        v[q] = t < rows * M ? src[t] : make_float2(0.f, 0.f);
+    }
+    if (src2) {
+#pragma unroll
+        for (int q = 0; q < LD; ++q) {
+            const int t = tid + q * Z::T;
+            const float2 w = t < rows * M ? src2[t] : make_float2(0.f, 0.f);
+            v[q] = make_float2(ca * v[q].x + cb * w.x, ca * v[q].y + cb * w.y);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < LD; ++q) {
+        const int t = tid + q * Z::T, r = t / M, m = t - r * M;
+        if (t < Z::R * M) A[r * Z::PITCH + m] = v[q];
+    }
+}
+
+// The thread's row of the block and its place in it.
+template <class Z>
+__device__ __forceinline__ void z_row(int& r, int& g, bool& act) {
+    const int lane = threadIdx.x & 31;
+    const int rw = lane / Z::G;
+    act = 32 % Z::G == 0 || rw < Z::RW;
+    r = (threadIdx.x >> 5) * Z::RW + (act ? rw : 0);
+    g = act ? lane - rw * Z::G : 0;
+}
+
+// four-step M-point transform of a row: v1[a][n1] = input N2 n1 + n2, n2 = g + G a, on
+// entry; output k1 + N1 k2, k1 = g + G a, in v2[a][k2]. S: the row's staging memory,
+// whose contents v1 already holds. t4: W_M^(n2 k1) at [k1][n2].
+template <class RG, bool INV>
+__device__ __forceinline__ void row_fft(float2* S, const float2* t4, int g, bool act, float2 (&v1)[RG::A1][RG::N1],
+                                        float2 (&v2)[RG::A2][RG::N2]) {
+    constexpr int N1 = RG::N1, N2 = RG::N2, G = RG::G;
+    __syncwarp();  // the row is in registers before S overwrites it
+#pragma unroll
+    for (int a = 0; a < RG::A1; ++a) {
+        const int n2 = g + G * a;
+        dft_reg<N1, INV>(v1[a]);
+#pragma unroll
+        for (int k1 = 0; k1 < N1; ++k1) {
+            float2 v = v1[a][k1];
+            if (k1 > 0) {
+                float2 w = t4[k1 * N2 + n2];
+                if (INV) w.y = -w.y;
+                v = cmul(v, w);
+            }
+            if (act) S[k1 * (N2 + 1) + n2] = v;
+        }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int a = 0; a < RG::A2; ++a) {
+        const int k1 = g + G * a;
+#pragma unroll
+        for (int n2 = 0; n2 < N2; ++n2) v2[a][n2] = S[k1 * (N2 + 1) + n2];
+        dft_reg<N2, INV>(v2[a]);
+    }
+}
+
+template <class RG>
+__global__ void __launch_bounds__(ZReg<RG>::T) k_z_r2c_reg(const __grid_constant__ ZFwd p, int nrows, const float2* __restrict__ twN) {
+    using Z = ZReg<RG>;
+    constexpr int M = Z::M, N1 = RG::N1, N2 = RG::N2, G = RG::G, A2 = RG::A2;
+    extern __shared__ float2 sm[];
+    float2* tw = sm;               // split table
+    float2* t4 = tw + Z::SPLIT;    // four-step table
+    float2* A = t4 + (M + 1) / 2 * 2;  // [R][PITCH]
+    const int tid = threadIdx.x;
+    const int row0 = blockIdx.x * Z::R;
+    const int rows = min(Z::R, nrows - row0);
+    load_z_tables<Z, RG>(tw, t4, twN);
+    const float* in2 = p.b[blockIdx.y];
+    stage_rows<Z>(A, reinterpret_cast<const float2*>(p.a[blockIdx.y]) + (int64_t)row0 * M, rows,
+                  in2 ? reinterpret_cast<const float2*>(in2) + (int64_t)row0 * M : nullptr, p.ca, p.cb);
+    __syncthreads();
+    int r, g;
+    bool act;
+    z_row<Z>(r, g, act);
+    float2* Ar = A + r * Z::PITCH;
+    float2 v1[RG::A1][N1], v2[A2][N2];
+#pragma unroll
+    for (int a = 0; a < RG::A1; ++a)
+#pragma unroll
+        for (int n1 = 0; n1 < N1; ++n1) v1[a][n1] = Ar[N2 * n1 + g + G * a];
+    row_fft<RG, false>(Ar, t4, g, act, v1, v2);
+    // X_k = E_k + exp(-2 pi i k / N) O_k from Z_k and conj(Z_(M-k)). Z_(M-k) of the
+    // thread's k = g + G a + N1 k2 is, for g > 0, element (A2 - 1 - a, N2 - 1 - k2) of
+    // thread G - g; for g = 0 one of its own.
+    auto split = [&](float2 zk, float2 zc, int kk) {
+        zc.y = -zc.y;
+        const float2 e = cscale(cadd(zk, zc), 0.5f);
+        const float2 dd = csub(zk, zc);
+        const float2 o = make_float2(0.5f * dd.y, -0.5f * dd.x);  // -i/2 (zk - zc)
+        return cadd(e, cmul(tw[kk], o));
+    };
+    const int lane = tid & 31;
+    const int src = g == 0 ? lane : lane - g + (G - g);
+    const int row = row0 + r;
+    const bool st = act && r < rows;
+    float2* orow = p.out[blockIdx.y] + (int64_t)row * M;
+#pragma unroll
+    for (int a = 0; a < A2; ++a)
+#pragma unroll
+        for (int k2 = 0; k2 < N2; ++k2) {
+            float2 zp = a == 0 ? v2[0][(N2 - k2) % N2] : v2[(A2 - a) % A2][N2 - 1 - k2];
+            if constexpr (G > 1) {
+                const float2 mine = v2[A2 - 1 - a][N2 - 1 - k2];
+                const float px = __shfl_sync(0xffffffffu, mine.x, src), py = __shfl_sync(0xffffffffu, mine.y, src);
+                if (g > 0) zp = make_float2(px, py);
+            }
+            const int k = g + G * a + N1 * k2;
+            const float2 x = split(v2[a][k2], zp, k);
+            if (st) orow[k] = x;
+        }
+    if (st && g == 0) p.out[blockIdx.y][(int64_t)nrows * M + row] = split(v2[0][0], v2[0][0], M);
+}
+
+template <class RG>
+__global__ void __launch_bounds__(ZReg<RG>::T) k_z_c2r_reg(const __grid_constant__ ZInv p, int nrows, float scale,
+                                                             const float2* __restrict__ twN) {
+    using Z = ZReg<RG>;
+    constexpr int M = Z::M, N = Z::N, N1 = RG::N1, N2 = RG::N2, G = RG::G;
+    extern __shared__ float2 sm[];
+    float2* tw = sm;               // split table
+    float2* t4 = tw + Z::SPLIT;    // four-step table
+    float2* A = t4 + (M + 1) / 2 * 2;  // [R][PITCH]: the M + 1 inputs of each row
+    const int tid = threadIdx.x;
+    const int row0 = blockIdx.x * Z::R;
+    const int rows = min(Z::R, nrows - row0);
+    load_z_tables<Z, RG>(tw, t4, twN);
+    const float2* in = p.in[blockIdx.y];
+    static_assert(Z::R <= Z::T, "one Nyquist value a thread");
+    const float2 nyq = tid < rows ? in[(int64_t)nrows * M + row0 + tid] : make_float2(0.f, 0.f);
+    stage_rows<Z>(A, in + (int64_t)row0 * M, rows, nullptr, 1.f, 0.f);
+    if (tid < Z::R) A[tid * Z::PITCH + M] = nyq;
+    __syncthreads();
+    int r, g;
+    bool act;
+    z_row<Z>(r, g, act);
+    float2* Ar = A + r * Z::PITCH;
+    // z_k = E_k + i O_k with E, O from X_k and conj(X_(M-k))
+    float2 v1[RG::A1][N1], v2[RG::A2][N2];
+#pragma unroll
+    for (int a = 0; a < RG::A1; ++a)
+#pragma unroll
+        for (int n1 = 0; n1 < N1; ++n1) {
+            const int k = N2 * n1 + g + G * a;
+            float2 xk = Ar[k], xc = Ar[M - k];
+            if (k == 0) {  // X_0 and X_M: imaginary parts carry nothing for a real signal
+                xk.y = 0.f;
+                xc.y = 0.f;
+            }
+            xc.y = -xc.y;
+            const float2 e = cscale(cadd(xk, xc), 0.5f);
+            float2 w = tw[k];
+            w.y = -w.y;  // exp(+2 pi i k / N)
+            const float2 o = cmul(cscale(csub(xk, xc), 0.5f), w);
+            v1[a][n1] = make_float2(e.x - o.y, e.y + o.x);  // e + i o
+        }
+    row_fft<RG, true>(Ar, t4, g, act, v1, v2);
+    // the row from the four-step's registers straight to global memory
+    if (act && r < rows) {
+        const float sc = scale * 2.0f / (float)N;
+        const int64_t o = (int64_t)(row0 + r) * M;
+        float2* d1 = reinterpret_cast<float2*>(p.out[blockIdx.y]) + o;
+        if (!p.out2[blockIdx.y]) {
+#pragma unroll
+            for (int a = 0; a < RG::A2; ++a)
+#pragma unroll
+                for (int k2 = 0; k2 < N2; ++k2) d1[g + G * a + N1 * k2] = cscale(v2[a][k2], sc);
+        } else {
+            float2* d2 = reinterpret_cast<float2*>(p.out2[blockIdx.y]) + o;
+#pragma unroll
+            for (int a = 0; a < RG::A2; ++a)
+#pragma unroll
+                for (int k2 = 0; k2 < N2; ++k2) {
+                    const float2 v = cscale(v2[a][k2], sc);
+                    d1[g + G * a + N1 * k2] = cscale(v, p.s1);
+                    d2[g + G * a + N1 * k2] = cscale(v, p.s2);
+                }
+        }
+    }
+}
+
+// ----------------------------------------------------------------------------- plan launches
+
+// RG: the column plan of N, RZ: the row plan of N / 2.
+template <class RG, class RZ>
+struct Plan {
+    using Z = ZReg<RZ>;
+    static constexpr int N = RG::N;
+    static_assert(2 * RZ::N == N, "row plan of the same mesh");
+    static void z_r2c(const ZFwd& p, int batch, const float2* tw, cudaStream_t s) {
+        k_z_r2c_reg<RZ><<<dim3(nblocks(N * N, Z::R), batch), Z::T, Z::smem(), s>>>(p, N * N, tw);
+    }
+    static void z_c2r(const ZInv& p, int batch, float scale, const float2* tw, cudaStream_t s) {
+        k_z_c2r_reg<RZ><<<dim3(nblocks(N * N, Z::R), batch), Z::T, Z::smem(), s>>>(p, N * N, scale, tw);
+    }
+    static void col(const float2* in, const Side& si, float2* out, const Side& so, int64_t bs, int batch, bool inv,
+                    const float2* tw, cudaStream_t s) {
+        if (inv) k_col_reg<RG, true><<<col_grid<RG>(batch), RG::T, RG::smem_col(), s>>>(in, out, bs, si, so, tw);
+        else k_col_reg<RG, false><<<col_grid<RG>(batch), RG::T, RG::smem_col(), s>>>(in, out, bs, si, so, tw);
+    }
+    // the fused x-pass of a large mesh takes 8 columns a block: 16 would leave one block
+    // per SM (512^3 one-to-three: 922 -> 677 us); the plain passes keep 16 (231 against 252 us)
+    using RX = Reg<RG::N1, RG::N2, (N >= 384 ? 8 : 16)>;
+    template <int MODE>
+    static void x_mode(const XFused& p, const Side& si, const Side& so, int batch, const float2* tw, cudaStream_t s) {
+        k_x_reg<RX, MODE><<<col_grid<RX>(batch), RX::T, RX::smem_x(MODE), s>>>(p, si, so, tw);
+    }
+    static void x(int mode, const XFused& p, const Side& si, const Side& so, int batch, const float2* tw,
+                  cudaStream_t s) {
+        switch (mode) {
+            case X_1TO1: return x_mode<X_1TO1>(p, si, so, batch, tw, s);
+            case X_1TO3_ODD: return x_mode<X_1TO3_ODD>(p, si, so, batch, tw, s);
+            case X_3TO1_ODD: return x_mode<X_3TO1_ODD>(p, si, so, batch, tw, s);
+            case X_1TON: return x_mode<X_1TON>(p, si, so, batch, tw, s);
+            default: return x_mode<X_NTO1>(p, si, so, batch, tw, s);
+        }
+    }
+    static void each_kernel(void (*set)(void*, const void*, size_t), void* arg) {
+        set(arg, (const void*)k_z_r2c_reg<RZ>, Z::smem());
+        set(arg, (const void*)k_z_c2r_reg<RZ>, Z::smem());
+        set(arg, (const void*)k_col_reg<RG, true>, RG::smem_col());
+        set(arg, (const void*)k_col_reg<RG, false>, RG::smem_col());
+        set(arg, (const void*)k_x_reg<RX, X_1TO1>, RX::smem_x(X_1TO1));
+        set(arg, (const void*)k_x_reg<RX, X_1TO3_ODD>, RX::smem_x(X_1TO3_ODD));
+        set(arg, (const void*)k_x_reg<RX, X_3TO1_ODD>, RX::smem_x(X_3TO1_ODD));
+        set(arg, (const void*)k_x_reg<RX, X_1TON>, RX::smem_x(X_1TON));
+        set(arg, (const void*)k_x_reg<RX, X_NTO1>, RX::smem_x(X_NTO1));
+    }
+    static const FFTOps* ops() {
+        static const FFTOps o{z_r2c, z_c2r, col, x, each_kernel};
+        return &o;
+    }
+};
+
+}  // namespace
+}  // namespace pmr

@@ -1,0 +1,22 @@
+// FFT plans of the mesh sides 8, 12, 16, 18, 24, 32, 36, 48, 54, 64 (fft_kernels.cuh).
+#include "fft_kernels.cuh"
+
+namespace pmr {
+
+const FFTOps* fft_plans_0(int N) {
+    switch (N) {
+        case 8: return Plan<Reg<4, 2>, Reg<2, 2>>::ops();
+        case 12: return Plan<Reg<6, 2>, Reg<6, 1>>::ops();
+        case 16: return Plan<Reg<2, 8>, Reg<2, 4>>::ops();
+        case 18: return Plan<Reg<6, 3>, Reg<9, 1>>::ops();
+        case 24: return Plan<Reg<4, 6>, Reg<6, 2>>::ops();
+        case 32: return Plan<Reg<8, 4>, Reg<4, 4>>::ops();
+        case 36: return Plan<Reg<6, 6>, Reg<6, 3>>::ops();
+        case 48: return Plan<Reg<12, 4>, Reg<6, 4>>::ops();
+        case 54: return Plan<Reg<9, 6>, Reg<9, 3>>::ops();
+        case 64: return Plan<Reg<8, 8>, Reg<8, 4>>::ops();
+        default: return nullptr;
+    }
+}
+
+}  // namespace pmr

@@ -145,8 +145,14 @@ static int smooth_into(pmr_ctx* c, const float* in, double R_mpc, float* out) {
 
 // Forward residual: c->M holds M_NN. Leaves M_R in c->MR and r_s in c->rs.
 int residual_forward(pmr_ctx* c, const float* data, const pmr_anneal* an, double* L_res_dev) {
-    PMR_TRY(smooth_into(c, c->M, c->cfg.R_M, c->MR));
-    PMR_TRY(smooth_into(c, data, c->cfg.R_M, c->DR));
+    if (c->cfg.R_M > 0) {
+        const float* ins[2] = {c->M, data};
+        float* outs[2] = {c->MR, c->DR};
+        PMR_TRY(conv_each(c, ins, outs, gauss_mul(c, c->cfg.R_M), 2));
+    } else {
+        PMR_TRY(smooth_into(c, c->M, 0.0, c->MR));
+        PMR_TRY(smooth_into(c, data, 0.0, c->DR));
+    }
     k_log_residual<<<nblocks(c->N3, kRT), kRT, 0, c->stream>>>(c->MR, c->DR, c->N3, (float)c->cfg.mu_N,
                                                                 (float)an->M0, c->gm);
     PMR_TRY(check_launch(c, "log_residual"));

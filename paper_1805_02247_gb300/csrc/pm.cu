@@ -758,22 +758,6 @@ __global__ void k_adj_readout_direct(const float* __restrict__ G, const float* _
     for (int a = 0; a < 3; ++a) lam_x[a * np + i] = lx[a] + kick * g[a];
 }
 
-// disp = D0 psi, p = Gp0 psi (psi already in disp)
-__global__ void k_za_finish(float* __restrict__ disp, float* __restrict__ mom, int64_t n, float D0, float Gp0) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    float psi = disp[i];
-    disp[i] = D0 * psi;
-    mom[i] = Gp0 * psi;
-}
-
-// lam_psi = D0 lam_x + Gp0 lam_p
-__global__ void k_za_adj_combine(const float* __restrict__ lx, const float* __restrict__ lp, float* __restrict__ out,
-                                 int64_t n, float D0, float Gp0) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] = D0 * lx[i] + Gp0 * lp[i];
-}
-
 // ----------------------------------------------------------------------------- second-order LPT
 
 // S = phi_xx phi_yy + phi_xx phi_zz + phi_yy phi_zz - phi_xy^2 - phi_xz^2 - phi_yz^2
@@ -930,10 +914,10 @@ int density_slot(pmr_ctx* c, int s, const float* disp, float* delta, bool sort) 
 int za_ics(pmr_ctx* c, const float2* s_k, float* disp, float* mom) {
     Mul mul[3];
     for (int j = 0; j < 3; ++j) mul[j] = Mul{MUL_ODD, j, 1.0f, 0.f, 0};
+    // D0 psi and Gp0 psi from one transform
     float* outs[3] = {disp, disp + c->N3, disp + 2 * c->N3};
-    PMR_TRY(k_to_real(c, s_k, outs, mul, 3));
-    k_za_finish<<<nblocks(3 * c->N3, kT), kT, 0, c->stream>>>(disp, mom, 3 * c->N3, (float)c->D0, (float)c->Gp0);
-    return check_launch(c, "za_finish");
+    float* outs2[3] = {mom, mom + c->N3, mom + 2 * c->N3};
+    return k_to_real(c, s_k, outs, mul, 3, outs2, (float)c->D0, (float)c->Gp0);
 }
 
 namespace {
@@ -983,13 +967,11 @@ int lpt_adjoint(pmr_ctx* c, const float2* s_k, const float* lam_x, const float* 
     const int64_t N3 = c->N3;
     if (!have_H) PMR_TRY(lpt2_hessian(c, s_k));
     // mu = D2 lam_x + Gp2 lam_p; sigma = sum_j irfft(conj(-i k_j / k^2) rfft(mu_j))
-    k_za_adj_combine<<<nblocks(3 * N3, kT), kT, 0, c->stream>>>(lam_x, lam_p, c->F, 3 * N3, (float)c->D2_0,
-                                                                 (float)c->Gp2_0);
-    PMR_TRY(check_launch(c, "lpt2_adj_combine"));
     Mul mul[3];
     for (int j = 0; j < 3; ++j) mul[j] = Mul{MUL_ODD, j, 1.0f, 0.f, 0};
-    const float* mu[3] = {c->F, c->F + N3, c->F + 2 * N3};
-    PMR_TRY(conv_Nto1(c, mu, mul, 3, c->delta));
+    const float* lx[3] = {lam_x, lam_x + N3, lam_x + 2 * N3};
+    const float* lp[3] = {lam_p, lam_p + N3, lam_p + 2 * N3};
+    PMR_TRY(conv_Nto1(c, lx, lp, (float)c->D2_0, (float)c->Gp2_0, mul, 3, c->delta));
     k_lpt2_hess_grad<<<nblocks(N3, kT), kT, 0, c->stream>>>(c->delta, c->lpt_H, N3, c->lpt_G);
     PMR_TRY(check_launch(c, "lpt2_hess_grad"));
     // grad += sum_ij (k_i k_j / k^2) (w / N^3) rfft(G_ij)
@@ -1003,7 +985,7 @@ int lpt_adjoint(pmr_ctx* c, const float2* s_k, const float* lam_x, const float* 
             hm[t] = Mul{MUL_HESS, pr[0], inv_n3, 0.f, 1, pr[1]};
             gin[t] = c->lpt_G + (int64_t)(3 * h + t) * N3;
         }
-        PMR_TRY(real_to_k_add(c, gin, hm, 3, grad));
+        PMR_TRY(real_to_k(c, gin, nullptr, 1.f, 0.f, hm, 3, grad, true));
     }
     return PMR_OK;
 }
@@ -1016,15 +998,12 @@ int kick_drift(pmr_ctx* c, const float* F, const float* din, float* dout, float*
 
 // grad_s = sum_j conj(i k_j / k^2) (w / N^3) rfft(D0 lam_x_j + Gp0 lam_p_j)
 int za_adjoint(pmr_ctx* c, const float* lam_x, const float* lam_p, float2* grad) {
-    float* tmp = c->F;  // 3 meshes of scratch
-    k_za_adj_combine<<<nblocks(3 * c->N3, kT), kT, 0, c->stream>>>(lam_x, lam_p, tmp, 3 * c->N3, (float)c->D0,
-                                                                     (float)c->Gp0);
-    PMR_TRY(check_launch(c, "za_adj_combine"));
     Mul mul[3];
     const float inv_n3 = (float)(1.0 / (double)c->N3);
     for (int j = 0; j < 3; ++j) mul[j] = Mul{MUL_ODD, j, -inv_n3, 0.f, 1};
-    const float* ins[3] = {tmp, tmp + c->N3, tmp + 2 * c->N3};
-    return real_to_k(c, ins, mul, 3, grad);
+    const float* lx[3] = {lam_x, lam_x + c->N3, lam_x + 2 * c->N3};
+    const float* lp[3] = {lam_p, lam_p + c->N3, lam_p + 2 * c->N3};
+    return real_to_k(c, lx, lp, (float)c->D0, (float)c->Gp0, mul, 3, grad, false);
 }
 
 int pm_forward_impl(pmr_ctx* c, const float2* s_k) {
@@ -1079,7 +1058,7 @@ int pm_adjoint_impl(pmr_ctx* c, const float* gfin, float2* grad) {
         PMR_TRY(paint3_sorted(c, c->perm_all + (int64_t)s * N3, c->start_all + (int64_t)s * (N3 + 1),
                               c->sfrac_all + (int64_t)s * 3 * N3, c->lam_p, (float)c->kick[s], Gj));
         const float* gins[3] = {Gj[0], Gj[1], Gj[2]};
-        PMR_TRY(conv_Nto1(c, gins, fmT, 3, c->gm));
+        PMR_TRY(conv_Nto1(c, gins, nullptr, 1.f, 0.f, fmT, 3, c->gm));
         if (s == 0) {
             PMR_TRY(readout_grad(c, c->gm, d, N3, true, 1.0f, true, c->lam_x));
             break;
