@@ -130,19 +130,14 @@ struct Sizes {
 template <class F>
 void for_each_buffer(const pmr_config& cfg, pmr_ctx* c, F alloc) {
     const int64_t N = cfg.N, N3 = N * N * N, P = N / 2 + 1, NH = N * N * P;
-    const int64_t nb_scan = (N3 + 1023) / 1024;
     alloc((void**)(c ? &c->disp : nullptr), sizeof(float) * 3 * N3 * (cfg.nsteps + 1));
     alloc((void**)(c ? &c->mom : nullptr), sizeof(float) * 3 * N3);
     alloc((void**)(c ? &c->lam_x : nullptr), sizeof(float) * 3 * N3);
     alloc((void**)(c ? &c->lam_p : nullptr), sizeof(float) * 3 * N3);
-    alloc((void**)(c ? &c->keys : nullptr), sizeof(uint32_t) * N3);
     alloc((void**)(c ? &c->perm : nullptr), sizeof(uint32_t) * N3);
     alloc((void**)(c ? &c->cell_start : nullptr), sizeof(uint32_t) * (N3 + 1));
-    alloc((void**)(c ? &c->counts : nullptr), sizeof(uint32_t) * N3);
-    alloc((void**)(c ? &c->scan_part : nullptr), sizeof(uint32_t) * nb_scan);
-    alloc((void**)(c ? &c->long_list : nullptr), sizeof(uint32_t) * N3);
-    alloc((void**)(c ? &c->long_count : nullptr), sizeof(uint32_t) * 4);
-    alloc((void**)(c ? &c->sort_tmp : nullptr), sizeof(uint32_t) * N3);
+    alloc((void**)(c ? &c->rec : nullptr), sizeof(float4) * N3);
+    alloc((void**)(c ? &c->run_cnt : nullptr), sizeof(uint32_t) * sort_run_words(N3));
     alloc((void**)(c ? &c->perm_all : nullptr), sizeof(uint32_t) * N3 * (cfg.nsteps + 1));
     alloc((void**)(c ? &c->start_all : nullptr), sizeof(uint32_t) * (N3 + 1) * (cfg.nsteps + 1));
     alloc((void**)(c ? &c->sfrac : nullptr), sizeof(float) * 3 * N3);

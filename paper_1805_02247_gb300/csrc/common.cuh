@@ -165,14 +165,10 @@ struct pmr_ctx {
     int64_t fwd_id = 0;  // counts completed forward sweeps (pmr_forward_id)
 
     // cell sort
-    uint32_t* keys = nullptr;
     uint32_t* perm = nullptr;
     uint32_t* cell_start = nullptr;  // N3 + 1
-    uint32_t* counts = nullptr;      // N3
-    uint32_t* scan_part = nullptr;
-    uint32_t* long_list = nullptr;   // cells whose segment needs the block sort
-    uint32_t* long_count = nullptr;
-    uint32_t* sort_tmp = nullptr;    // N3 scratch for the block sort
+    float4* rec = nullptr;           // N3 particles binned by run (pack_rec in pm.cu)
+    uint32_t* run_cnt = nullptr;     // counts, cursors and starts of the sort's runs (sort_run_words)
     // per-step sort of the path's positions, kept from the forward sweep for the
     // adjoint: slot s holds perm [N3] and cell offsets [N3 + 1] of x_s, s = 0..nsteps
     uint32_t* perm_all = nullptr;
@@ -274,6 +270,13 @@ int real_to_k(pmr_ctx* c, const float* const* in, const float* const* in2, float
 // positions are either explicit absolute positions (lattice == false) or
 // lattice + displacement (lattice == true; q from the particle index)
 int cell_sort(pmr_ctx* c, const float* pos, int64_t np, bool lattice, uint32_t* keys_out);
+constexpr int kRunPad = 32;  // words between two run counters: one to a line, so that L2 serves them side by side
+int sort_run_log(int64_t ncell);  // log2 of the cells in one run of the sort
+// words of pmr_ctx::run_cnt for a mesh of ncell cells
+inline int64_t sort_run_words(int64_t ncell) {
+    const int rs_log = sort_run_log(ncell);
+    return (2 * kRunPad + 1) * ((ncell + (1 << rs_log) - 1) >> rs_log) + 1;
+}
 int paint(pmr_ctx* c, const float* pos, int64_t np, bool lattice, const float* mass, int nmass,
           float scale, float offset, float* const* rho);
 int readout(pmr_ctx* c, const float* field, const float* pos, int64_t np, bool lattice, float* out);
@@ -289,7 +292,7 @@ int lpt_adjoint(pmr_ctx* c, const float2* s_k, const float* lam_x, const float* 
 int pm_forward_impl(pmr_ctx* c, const float2* s_k);
 int pm_adjoint_impl(pmr_ctx* c, const float* gfin, float2* grad);  // gfin: gradient w.r.t. the final density
 int density_from(pmr_ctx* c, const float* disp, float* delta);
-// sfrac (nullable): also write the particles' fractional offsets in sorted order, [3][np]
+// sfrac: the particles' fractional offsets in sorted order, [3][np]
 int cell_sort_into(pmr_ctx* c, const float* pos, int64_t np, bool lattice, uint32_t* keys_out, uint32_t* perm,
                    uint32_t* start, float* sfrac);
 // sfrac (nullable): the offsets written by the sort that produced perm/start

@@ -21,16 +21,12 @@ constexpr size_t kAlign = 256;
 constexpr size_t up(size_t b) { return (b + kAlign - 1) / kAlign * kAlign; }
 
 // Scratch regions (bytes), each 256-byte aligned.
-constexpr size_t kKeys = up(4 * kMaxParticles);
 constexpr size_t kPerm = up(4 * kMaxParticles);
-constexpr size_t kTmp = up(4 * kMaxParticles);
 constexpr size_t kStart = up(4 * (kMaxCells + 1));
-constexpr size_t kCounts = up(4 * kMaxCells);
-constexpr size_t kLong = up(4 * kMaxCells);
-constexpr size_t kPart = up(4 * ((kMaxCells + 1023) / 1024));
-constexpr size_t kLongCount = up(16);
+constexpr size_t kRec = up(16 * kMaxParticles);
+constexpr size_t kRuns = up(4 * ((2 * pmr::kRunPad + 1) * ((kMaxCells >> 9) + 1) + 1));  // runs of 512 cells at these sizes
 constexpr size_t kFrac = up(4 * 3 * kMaxParticles);  // sorted fractional offsets, as pmr_paint uses them
-constexpr size_t kScratchBytes = kKeys + kPerm + kTmp + kStart + kCounts + kLong + kPart + kLongCount + kFrac;
+constexpr size_t kScratchBytes = kPerm + kStart + kRec + kRuns + kFrac;
 
 // Every GPU that loads the library holds this array until the process exits.
 static __device__ __align__(256) unsigned char g_paint_scratch[kScratchBytes];
@@ -78,17 +74,15 @@ extern "C" int pmr_paint_noalloc(int N, const float* x, int64_t np, const float*
     c.N = N;
     c.N3 = (int64_t)N * N * N;
     unsigned char* p = base;
-    c.keys = reinterpret_cast<uint32_t*>(p); p += kKeys;
     c.perm = reinterpret_cast<uint32_t*>(p); p += kPerm;
-    c.sort_tmp = reinterpret_cast<uint32_t*>(p); p += kTmp;
     c.cell_start = reinterpret_cast<uint32_t*>(p); p += kStart;
-    c.counts = reinterpret_cast<uint32_t*>(p); p += kCounts;
-    c.long_list = reinterpret_cast<uint32_t*>(p); p += kLong;
-    c.scan_part = reinterpret_cast<uint32_t*>(p); p += kPart;
-    c.long_count = reinterpret_cast<uint32_t*>(p); p += kLongCount;
+    c.rec = reinterpret_cast<float4*>(p); p += kRec;
+    c.run_cnt = reinterpret_cast<uint32_t*>(p); p += kRuns;
     c.sfrac = reinterpret_cast<float*>(p);
+    if ((size_t)pmr::sort_run_words(c.N3) * 4 > kRuns)
+        return pmr::fail(nullptr, PMR_EINVAL, "pmr_paint_noalloc: the fixed array does not hold this mesh's runs");
 
-    // cell_sort clears the histogram and the long-segment counter itself;
+    // cell_sort clears the run counters itself;
     // every other region is fully written before it is read.
     int rc = pmr::cell_sort(&c, x, np, false, nullptr);
     if (rc == PMR_OK) {

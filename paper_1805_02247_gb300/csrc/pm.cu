@@ -37,31 +37,41 @@ __device__ __forceinline__ void lattice_of(uint32_t i, const FastDiv& fN, int q[
     q[1] = (int)(t - (uint32_t)q[0] * fN.d);
 }
 
-__device__ __forceinline__ Cell cell_of(const float* __restrict__ pos, int64_t np, int64_t i, bool lattice, int N,
-                                        const FastDiv& fN) {
+// cell and offset of a particle at u: a displacement from its lattice point (i
+// is its index) or an absolute position
+__device__ __forceinline__ Cell cell_at(const float u[3], uint32_t i, bool lattice, int N, const FastDiv& fN) {
     Cell c;
     if (lattice) {
         int q[3];
-        lattice_of((uint32_t)i, fN, q);
+        lattice_of(i, fN, q);
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            float u = pos[a * np + i];
-            float f = floorf(u);
-            c.d[a] = u - f;
-            int ii = (q[a] + (int)f) % N;
-            c.i[a] = ii < 0 ? ii + N : ii;
+            const float f = floorf(u[a]);
+            c.d[a] = u[a] - f;
+            int ii = q[a] + (int)f;
+            if ((uint32_t)ii >= (uint32_t)N) {  // the division only for particles that left the box
+                ii %= N;
+                ii = ii < 0 ? ii + N : ii;
+            }
+            c.i[a] = ii;
         }
     } else {
         const float n = (float)N;
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            float w = wrap_pos(pos[a * np + i], n);
-            float f = floorf(w);
+            const float w = wrap_pos(u[a], n);
+            const float f = floorf(w);
             c.i[a] = (int)f;
             c.d[a] = w - f;
         }
     }
     return c;
+}
+
+__device__ __forceinline__ Cell cell_of(const float* __restrict__ pos, int64_t np, int64_t i, bool lattice, int N,
+                                        const FastDiv& fN) {
+    const float u[3] = {pos[i], pos[np + i], pos[2 * np + i]};
+    return cell_at(u, (uint32_t)i, lattice, N, fN);
 }
 
 __device__ __forceinline__ uint32_t key_of(const Cell& c, int N) {
@@ -99,145 +109,141 @@ __device__ __forceinline__ void dwgt(const Cell& c, int o, float g[3]) {
 
 // ----------------------------------------------------------------------------- sort
 
-__global__ void k_keys(const float* __restrict__ pos, int64_t np, bool lattice, int N, FastDiv fN, uint32_t* __restrict__ keys,
-                       uint32_t* __restrict__ counts, uint32_t* __restrict__ rank) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= np) return;
-    uint32_t k = key_of(cell_of(pos, np, i, lattice, N, fN), N);
-    keys[i] = k;
-    // the particle's slot in its cell (arbitrary among the cell's particles;
-    // k_seg_fix restores ascending particle index)
-    rank[i] = atomicAdd(&counts[k], 1u);
-}
+// Counting sort by cell key, stable by particle index, through runs of
+// consecutive cells: k_run_count counts the particles of every run, k_run_scan
+// turns the counts into offsets, k_run_place writes each particle's offsets, index and
+// local cell into its run (in any order) and k_run_sort, a block per run, sorts its
+// particles by (cell, index) in shared memory and writes the cell offsets, the
+// permutation and the fractional CIC offsets in sorted order. A warp's particles
+// fall in a few runs, so the global counters take a few atomics a warp, not one
+// a particle, and the position is read by streaming passes only.
 
-// Exclusive scan of the cell counts, reduce-then-scan: k_scan_reduce sums each
-// block's kScanBlock counts, k_scan_part scans the block sums (one block),
-// k_scan_apply scans each block from its offset.
-constexpr int kScanT = 256, kScanPerT = 16, kScanBlock = kScanT * kScanPerT;
+// lanes of the warp in the same run; UINT_MAX: no particle
+__device__ __forceinline__ uint32_t same_run(uint32_t run) { return __match_any_sync(0xffffffffu, run); }
+constexpr uint32_t kNoRun = 0xffffffffu;
+constexpr int kBinP = 4;  // particles per thread of the two binning passes, blockDim apart
 
-__device__ __forceinline__ uint32_t warp_sum_u32(uint32_t v) {
+__global__ void __launch_bounds__(kT) k_run_count(const float* __restrict__ pos, int64_t np, bool lattice, int N,
+                                                  FastDiv fN, int rs_log, uint32_t* __restrict__ keys,
+                                                  uint32_t* __restrict__ cnt) {
+    const int64_t i0 = (int64_t)blockIdx.x * (kT * kBinP) + threadIdx.x;
+    float u[kBinP][3];
 #pragma unroll
-    for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
-    return v;
-}
-
-__global__ void __launch_bounds__(kScanT) k_scan_reduce(const uint32_t* __restrict__ in, int64_t n,
-                                                        uint32_t* __restrict__ part) {
-    __shared__ uint32_t wsum[kScanT / 32];
-    const int64_t b0 = (int64_t)blockIdx.x * kScanBlock;
-    uint32_t s = 0;
+    for (int q = 0; q < kBinP; ++q) {
+        const int64_t i = i0 + q * kT;
+        if (i < np)
 #pragma unroll
-    for (int k = 0; k < kScanPerT; ++k) {
-        const int64_t i = b0 + k * kScanT + threadIdx.x;
-        if (i < n) s += in[i];
+            for (int a = 0; a < 3; ++a) u[q][a] = pos[a * np + i];
     }
-    s = warp_sum_u32(s);
-    if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        uint32_t t = threadIdx.x < kScanT / 32 ? wsum[threadIdx.x] : 0u;
-        t = warp_sum_u32(t);
-        if (threadIdx.x == 0) part[blockIdx.x] = t;
+#pragma unroll
+    for (int q = 0; q < kBinP; ++q) {
+        const int64_t i = i0 + q * kT;
+        uint32_t run = kNoRun;
+        if (i < np) {
+            const uint32_t k = key_of(cell_at(u[q], (uint32_t)i, lattice, N, fN), N);
+            if (keys) keys[i] = k;
+            run = k >> rs_log;
+        }
+        const uint32_t m = same_run(run);
+        if (run != kNoRun && (m & ((1u << (threadIdx.x & 31)) - 1u)) == 0) atomicAdd(&cnt[run * kRunPad], (uint32_t)__popc(m));
     }
 }
 
-// Phase 2: exclusive scan of the block totals by one block (serial chunks).
-constexpr int kScanPartT = 1024;
-__global__ void __launch_bounds__(kScanPartT) k_scan_part(uint32_t* __restrict__ part, int nb,
-                                                         uint32_t* __restrict__ total_out) {
-    __shared__ uint32_t carry;
-    __shared__ uint32_t wsum[kScanPartT / 32];
-    if (threadIdx.x == 0) carry = 0;
-    __syncthreads();
+// Exclusive scan of the run counts: start[run], start[nruns] = np, and the placing
+// pass's cursors. A block owns kScanT runs and adds up all counts before them itself
+// (a few thousand reads that hit L2, side by side in all blocks).
+constexpr int kScanT = 1024;
+__global__ void __launch_bounds__(kScanT) k_run_scan(const uint32_t* __restrict__ cnt, int nruns,
+                                                     uint32_t* __restrict__ start, uint32_t* __restrict__ cursor) {
+    __shared__ uint32_t wsum[kScanT / 32], wpre[kScanT / 32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int b0 = 0; b0 < nb; b0 += kScanPartT) {
-        int idx = b0 + threadIdx.x;
-        uint32_t v = idx < nb ? part[idx] : 0u, inc = v;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            uint32_t t = __shfl_up_sync(0xffffffffu, inc, d);
-            if (lane >= d) inc += t;
-        }
-        if (lane == 31) wsum[wid] = inc;
-        __syncthreads();
-        if (wid == 0) {
-            uint32_t t = (lane < kScanPartT / 32) ? wsum[lane] : 0u, ti = t;
-#pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                uint32_t u = __shfl_up_sync(0xffffffffu, ti, d);
-                if (lane >= d) ti += u;
-            }
-            if (lane < kScanPartT / 32) wsum[lane] = ti - t;
-        }
-        __syncthreads();
-        uint32_t ex = carry + wsum[wid] + inc - v;
-        if (idx < nb) part[idx] = ex;
-        __syncthreads();
-        if (threadIdx.x == kScanPartT - 1) carry = ex + v;
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) *total_out = carry;
-}
-
-// shared-memory index with one padding word per 32, so a thread's run of
-// kScanPerT consecutive elements and a warp's run of 32 are both conflict-free
-__device__ __forceinline__ int scan_sidx(int e) { return e + (e >> 5); }
-
-__global__ void __launch_bounds__(kScanT) k_scan_apply(const uint32_t* __restrict__ in, int64_t n,
-                                                       const uint32_t* __restrict__ part, uint32_t* __restrict__ out) {
-    __shared__ uint32_t tile[kScanBlock + kScanBlock / 32];
-    __shared__ uint32_t wtot[kScanT / 32];
-    const int64_t b0 = (int64_t)blockIdx.x * kScanBlock;
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-#pragma unroll
-    for (int k = 0; k < kScanPerT; ++k) {
-        const int e = k * kScanT + tid;
-        tile[scan_sidx(e)] = b0 + e < n ? in[b0 + e] : 0u;
-    }
-    __syncthreads();
-    uint32_t v[kScanPerT], s = 0;
-#pragma unroll
-    for (int k = 0; k < kScanPerT; ++k) {
-        v[k] = tile[scan_sidx(tid * kScanPerT + k)];
-        s += v[k];
-    }
-    uint32_t inc = s;
+    const int b0 = blockIdx.x * kScanT, i = b0 + threadIdx.x;
+    const uint32_t v = i < nruns ? cnt[i * kRunPad] : 0u;
+    uint32_t pre = 0;
+#pragma unroll 8
+    for (int q = threadIdx.x; q < b0; q += kScanT) pre += cnt[q * kRunPad];
+    uint32_t inc = v;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
-        const uint32_t t = __shfl_up_sync(0xffffffffu, inc, d);
-        if (lane >= d) inc += t;
+        const uint32_t o = __shfl_up_sync(0xffffffffu, inc, d);
+        if (lane >= d) inc += o;
+        pre += __shfl_xor_sync(0xffffffffu, pre, d);
     }
-    if (lane == 31) wtot[wid] = inc;
+    if (lane == 31) wsum[wid] = inc;
+    if (lane == 0) wpre[wid] = pre;
     __syncthreads();
-    if (wid == 0) {
-        uint32_t t = lane < kScanT / 32 ? wtot[lane] : 0u, ti = t;
+    uint32_t w = lane < wid ? wsum[lane] : 0u;  // the warps before this one
+    w += wpre[lane];                             // and the blocks before this one
 #pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const uint32_t u = __shfl_up_sync(0xffffffffu, ti, d);
-            if (lane >= d) ti += u;
-        }
-        if (lane < kScanT / 32) wtot[lane] = ti - t;
-    }
-    __syncthreads();
-    uint32_t run = part[blockIdx.x] + wtot[wid] + inc - s;
-#pragma unroll
-    for (int k = 0; k < kScanPerT; ++k) {
-        tile[scan_sidx(tid * kScanPerT + k)] = run;
-        run += v[k];
-    }
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < kScanPerT; ++k) {
-        const int e = k * kScanT + tid;
-        if (b0 + e < n) out[b0 + e] = tile[scan_sidx(e)];
+    for (int d = 16; d > 0; d >>= 1) w += __shfl_xor_sync(0xffffffffu, w, d);
+    const uint32_t ex = w + inc - v;
+    if (i < nruns) {
+        start[i] = ex;
+        cursor[i * kRunPad] = ex;
+        if (i == nruns - 1) start[nruns] = ex + v;
     }
 }
 
-__global__ void k_scatter(const uint32_t* __restrict__ keys, const uint32_t* __restrict__ rank, int64_t np,
-                          const uint32_t* __restrict__ start, uint32_t* __restrict__ perm) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= np) return;
-    perm[start[keys[i]] + rank[i]] = (uint32_t)i;
+// A binned particle in 16 bytes: its offsets, index (27 bits) and cell within the run
+// (11 bits). An offset lies in [0, 1], so the top two bits of its float are free; a NaN,
+// whose top bits are overwritten, reads back as a value above 1 and is NaN again.
+__device__ __forceinline__ float4 pack_rec(const float d[3], uint32_t i, uint32_t l) {
+    const uint32_t m = 0x3fffffffu;
+    return make_float4(__uint_as_float((__float_as_uint(d[0]) & m) | ((l >> 5) & 3u) << 30),
+                       __uint_as_float((__float_as_uint(d[1]) & m) | ((l >> 7) & 3u) << 30),
+                       __uint_as_float((__float_as_uint(d[2]) & m) | ((l >> 9) & 3u) << 30),
+                       __uint_as_float(i | (l & 31u) << 27));
+}
+__device__ __forceinline__ uint32_t rec_cell(const float4& r) {
+    return __float_as_uint(r.w) >> 27 | (__float_as_uint(r.x) >> 30) << 5 | (__float_as_uint(r.y) >> 30) << 7 |
+           (__float_as_uint(r.z) >> 30) << 9;
+}
+__device__ __forceinline__ uint32_t rec_index(const float4& r) { return __float_as_uint(r.w) & 0x7ffffffu; }
+__device__ __forceinline__ float rec_offset(float x) {
+    const uint32_t b = __float_as_uint(x) & 0x3fffffffu;
+    return b > 0x3f800000u ? __uint_as_float(0x7fc00000u) : __uint_as_float(b);
+}
+
+// rec[slot] = the particle, slots of a run handed out by its cursor in any order
+__global__ void __launch_bounds__(kT) k_run_place(const float* __restrict__ pos, int64_t np, bool lattice, int N,
+                                                  FastDiv fN, int rs_log, uint32_t* __restrict__ cursor,
+                                                  float4* __restrict__ rec) {
+    const int64_t i0 = (int64_t)blockIdx.x * (kT * kBinP) + threadIdx.x;
+    const int lane = threadIdx.x & 31;
+    float u[kBinP][3];
+#pragma unroll
+    for (int q = 0; q < kBinP; ++q) {
+        const int64_t i = i0 + q * kT;
+        if (i < np)
+#pragma unroll
+            for (int a = 0; a < 3; ++a) u[q][a] = pos[a * np + i];
+    }
+    uint32_t base[kBinP], m[kBinP], key[kBinP];
+#pragma unroll
+    for (int q = 0; q < kBinP; ++q) {  // every atomic of the thread in flight before the first is used
+        const int64_t i = i0 + q * kT;
+        uint32_t run = kNoRun;
+        if (i < np) {
+            const Cell c = cell_at(u[q], (uint32_t)i, lattice, N, fN);
+            key[q] = key_of(c, N);
+            run = key[q] >> rs_log;
+#pragma unroll
+            for (int a = 0; a < 3; ++a) u[q][a] = c.d[a];
+        }
+        m[q] = same_run(run);
+        base[q] = 0;
+        if (run != kNoRun && (m[q] & ((1u << lane) - 1u)) == 0)
+            base[q] = atomicAdd(&cursor[run * kRunPad], (uint32_t)__popc(m[q]));
+    }
+#pragma unroll
+    for (int q = 0; q < kBinP; ++q) {
+        const int64_t i = i0 + q * kT;
+        const uint32_t b = __shfl_sync(0xffffffffu, base[q], __ffs(m[q]) - 1);
+        if (i < np) {
+            const uint32_t slot = b + __popc(m[q] & ((1u << lane) - 1u));
+            rec[slot] = pack_rec(u[q], (uint32_t)i, key[q] & ((1u << rs_log) - 1u));
+        }
+    }
 }
 
 // out[m][j] = in[m][perm[j]]: per-particle values into the order of a sort
@@ -251,18 +257,11 @@ __global__ void k_permute3(const uint32_t* __restrict__ perm, const float* __res
     out[2 * np + j] = in[2 * np + i];
 }
 
-// Ascending particle index inside every cell segment (the scatter leaves it
-// arbitrary), then, with sfrac, every particle's fractional CIC offsets in the
-// sorted order: sfrac[a][j] of particle perm[j] (the float32 values cell_of
-// gives). A block owns kFixCells consecutive cells, whose particles are one
-// contiguous run of perm: the run is staged in shared memory, segments of up to
-// kSegThread particles are insertion-sorted by one thread each, up to
-// kSegWarp by one warp (warp_seg_sort in registers up to 32, seg_sort<true>
-// in shared memory beyond), longer ones (crowded cells of a clustered field)
-// by the whole block with seg_sort<false>, and
-// the run is written back with coalesced stores. A run longer than kFixCap is
-// listed in ovf for k_seg_fix_big, which does the same in global memory.
-constexpr int kFixCells = 512, kFixT = 256, kFixCap = 5120, kSegThread = 8, kSegWarp = 512;
+// Cells with up to kSegThread particles are ordered by comparison when they are
+// written, longer segments are sorted first: up to kSegWarp by one warp
+// (warp_seg_sort in registers up to 32, seg_sort<true> beyond), crowded cells of
+// a clustered field by the whole block with seg_sort<false>.
+constexpr int kSegThread = 8, kSegWarp = 512;
 
 // Sorts a[0, len) ascending with every thread of the block, or with the 32
 // lanes of the calling warp when WARP (a bitonic network over the next power of
@@ -304,18 +303,6 @@ __device__ void seg_sort(uint32_t* a, int len) {
     }
 }
 
-__device__ __forceinline__ void write_sorted(uint32_t i, int64_t j, const float* __restrict__ pos, int64_t np,
-                                             bool lattice, int N, const FastDiv& fN, uint32_t* __restrict__ perm,
-                                             float* __restrict__ sfrac) {
-    perm[j] = i;
-    if (sfrac) {
-        const Cell cl = cell_of(pos, np, i, lattice, N, fN);
-        sfrac[j] = cl.d[0];
-        sfrac[np + j] = cl.d[1];
-        sfrac[2 * np + j] = cl.d[2];
-    }
-}
-
 // Sorts a[0, len), len <= 32, ascending with the 32 lanes of a warp: a bitonic
 // network on one value per lane (UINT_MAX padding) through shuffles.
 __device__ __forceinline__ void warp_seg_sort(uint32_t* a, int len) {
@@ -333,129 +320,172 @@ __device__ __forceinline__ void warp_seg_sort(uint32_t* a, int len) {
     if (lane < len) a[lane] = v;
 }
 
-__global__ void __launch_bounds__(kFixT) k_seg_fix(const uint32_t* __restrict__ start, uint32_t* __restrict__ perm,
-                                                   int64_t ncell, const float* __restrict__ pos, int64_t np,
-                                                   bool lattice, int N, FastDiv fN, float* __restrict__ sfrac,
-                                                   uint32_t* __restrict__ ovf, uint32_t* __restrict__ novf) {
-    __shared__ uint32_t buf[kFixCap];
-    __shared__ uint32_t sst[kFixCells + 1];
-    __shared__ uint32_t longs[kFixCells];
-    __shared__ uint32_t meds[kFixCells];
-    __shared__ int nlong, nmed;
-    const int tid = threadIdx.x;
-    const int64_t c0 = (int64_t)blockIdx.x * kFixCells;
-    const int nc = (int)min((int64_t)kFixCells, ncell - c0);
-    for (int t = tid; t <= nc; t += kFixT) sst[t] = start[c0 + t];
-    if (tid == 0) nlong = nmed = 0;
+// Run sizes: RS cells and T threads a run. 2048 cells keep the binned pieces long;
+// small meshes take 512 so that the runs fill the chip. K: particles a thread keeps in
+// registers (runs of up to K T particles, 1.5 times one a cell and more, take the
+// path on registers). CAP: particles a longer run may list in shared memory.
+template <int RS_LOG>
+struct RunCfg {
+    static constexpr int RS = 1 << RS_LOG, T = RS_LOG >= 11 ? 512 : 256, PER = RS / T, CAP = 11 * RS / 4;
+    static constexpr int K = 6;
+    static_assert(K * T >= 3 * RS / 2 && K * T <= 4096 && RS <= 2048 && CAP >= K * T / 2, "packing of lr");
+};
+
+// The sort of one run's particles, rec[s0, s1). 16 bytes a particle in, 16 out and 4 a
+// cell; the phases of a block (records, cell counts, scan, index lists, output) follow
+// each other through barriers, so a thread keeps all its records in flight and in
+// registers. Bound by instructions and shared memory.
+template <int RS_LOG>
+__global__ void __launch_bounds__(RunCfg<RS_LOG>::T, 1024 / RunCfg<RS_LOG>::T)
+    k_run_sort(const float4* __restrict__ rec, const uint32_t* __restrict__ rstart, int64_t ncell, int64_t np,
+               uint32_t* __restrict__ start, uint32_t* perm, float* __restrict__ sfrac) {
+    using R = RunCfg<RS_LOG>;
+    __shared__ uint32_t cst[R::RS + 1];  // cell counts, then their exclusive scan
+    __shared__ uint32_t sidx[R::CAP > R::K * R::T ? R::CAP : R::K * R::T];  // particle indices by cell
+    __shared__ uint16_t segs[R::RS];  // cells to sort: by a warp from the front, by the block from the back
+    __shared__ uint32_t wsum[R::T / 32];
+    __shared__ int nwarp, nblock;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int64_t c0 = (int64_t)blockIdx.x << RS_LOG;
+    const int nc = (int)min((int64_t)R::RS, ncell - c0);
+    const uint32_t s0 = rstart[blockIdx.x];
+    const int n = (int)(rstart[blockIdx.x + 1] - s0);
+    const bool in_regs = n <= R::K * R::T;
+    const bool big = n > R::CAP && !in_regs;  // the index list is perm itself
+    uint32_t* seg = big ? perm + s0 : sidx;
+    float4 r[R::K];     // the thread's particles
+    uint32_t lr[R::K];  // local cell, and the particle's slot in it << 12
+    if (in_regs)
+#pragma unroll
+        for (int k = 0; k < R::K; ++k)
+            if (tid + k * R::T < n) r[k] = rec[s0 + tid + k * R::T];
+    for (int l = tid; l < R::RS; l += R::T) cst[l] = 0;
+    if (tid == 0) nwarp = nblock = 0;
     __syncthreads();
-    const uint32_t s0 = sst[0];
-    const int n = (int)(sst[nc] - s0);
-    if (n > kFixCap) {
-        if (tid == 0) ovf[atomicAdd(novf, 1u)] = blockIdx.x;
+    if (in_regs) {
+#pragma unroll
+        for (int k = 0; k < R::K; ++k)
+            if (tid + k * R::T < n) {
+                const uint32_t l = rec_cell(r[k]);
+                lr[k] = l | atomicAdd(&cst[l], 1u) << 12;
+            }
+    } else {
+        for (int j = tid; j < n; j += R::T) atomicAdd(&cst[rec_cell(rec[s0 + j])], 1u);
+    }
+    __syncthreads();
+    {
+        uint32_t v[R::PER], s = 0;
+#pragma unroll
+        for (int k = 0; k < R::PER; ++k) {
+            v[k] = cst[tid * R::PER + k];
+            s += v[k];
+        }
+        uint32_t inc = s;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t o = __shfl_up_sync(0xffffffffu, inc, d);
+            if (lane >= d) inc += o;
+        }
+        if (lane == 31) wsum[wid] = inc;
+        __syncthreads();
+        uint32_t run = inc - s;
+        for (int w = 0; w < wid; ++w) run += wsum[w];
+#pragma unroll
+        for (int k = 0; k < R::PER; ++k) {
+            const int l = tid * R::PER + k;
+            cst[l] = run;
+            if (v[k] > (uint32_t)kSegWarp) segs[R::RS - 1 - atomicAdd(&nblock, 1)] = (uint16_t)l;
+            else if (v[k] > (uint32_t)kSegThread) segs[atomicAdd(&nwarp, 1)] = (uint16_t)l;
+            run += v[k];
+        }
+        if (tid == R::T - 1) cst[R::RS] = run;
+    }
+    __syncthreads();
+    for (int l = tid; l < nc; l += R::T) start[c0 + l] = s0 + cst[l];
+    if (tid == 0 && c0 + nc == ncell) start[ncell] = s0 + (uint32_t)n;
+    // indices into their cells' segments
+    if (in_regs) {
+#pragma unroll
+        for (int k = 0; k < R::K; ++k)
+            if (tid + k * R::T < n) sidx[cst[lr[k] & 0xfffu] + (lr[k] >> 12)] = rec_index(r[k]);
+    } else {
+        __syncthreads();
+        for (int j = tid; j < n; j += R::T) {
+            const float4 q = rec[s0 + j];
+            seg[atomicAdd(&cst[rec_cell(q)], 1u)] = rec_index(q);
+        }
+        __syncthreads();  // cst[l] is now the end of cell l, the start of l + 1: shift it back
+        uint32_t e[R::PER];
+#pragma unroll
+        for (int k = 0; k < R::PER; ++k) e[k] = tid * R::PER + k > 0 ? cst[tid * R::PER + k - 1] : 0u;
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < R::PER; ++k) cst[tid * R::PER + k] = e[k];
+    }
+    __syncthreads();
+    for (int q = wid; q < nwarp; q += R::T / 32) {
+        const uint32_t a = cst[segs[q]];
+        const int len = (int)(cst[segs[q] + 1] - a);
+        if (len <= 32) warp_seg_sort(seg + a, len);
+        else seg_sort<true>(seg + a, len);
+    }
+    if (nblock > 0) {
+        __syncthreads();
+        for (int q = 0; q < nblock; ++q) {
+            const int l = segs[R::RS - 1 - q];
+            seg_sort<false>(seg + cst[l], (int)(cst[l + 1] - cst[l]));
+        }
+    }
+    if (nwarp > 0) __syncthreads();
+    // A particle's place: among up to kSegThread by counting the smaller indices of its
+    // cell, in a sorted segment by bisection.
+    auto place = [&](uint32_t l, uint32_t i) {
+        uint32_t a = cst[l], e = cst[l + 1];
+        if (e - a > (uint32_t)kSegThread || big) {
+            while (e - a > 1) {
+                const uint32_t mid = (a + e) >> 1;
+                if (seg[mid] <= i) a = mid;
+                else e = mid;
+            }
+        } else if (e - a > 1) {
+            uint32_t less = 0;
+            for (uint32_t p = a; p < e; ++p) less += seg[p] < i ? 1u : 0u;
+            a += less;
+        }
+        return s0 + a;
+    };
+    if (in_regs) {
+#pragma unroll
+        for (int k = 0; k < R::K; ++k)
+            if (tid + k * R::T < n) {
+                const uint32_t i = rec_index(r[k]), p = place(lr[k] & 0xfffu, i);
+                perm[p] = i;
+                sfrac[p] = rec_offset(r[k].x);
+                sfrac[np + p] = rec_offset(r[k].y);
+                sfrac[2 * np + p] = rec_offset(r[k].z);
+            }
         return;
     }
-    for (int j = tid; j < n; j += kFixT) buf[j] = perm[s0 + j];
-    __syncthreads();
-    for (int cl = tid; cl < nc; cl += kFixT) {
-        const int a = (int)(sst[cl] - s0), e = (int)(sst[cl + 1] - s0);
-        if (e - a <= 1) continue;
-        if (e - a > kSegWarp) {
-            longs[atomicAdd(&nlong, 1)] = (uint32_t)cl;
-            continue;
-        }
-        if (e - a > kSegThread) {  // one warp per segment, below
-            meds[atomicAdd(&nmed, 1)] = (uint32_t)cl;
-            continue;
-        }
-        for (int p = a + 1; p < e; ++p) {
-            const uint32_t v = buf[p];
-            int q = p - 1;
-            while (q >= a && buf[q] > v) {
-                buf[q + 1] = buf[q];
-                --q;
-            }
-            buf[q + 1] = v;
-        }
-    }
-    __syncthreads();
-    for (int mi = tid >> 5; mi < nmed; mi += kFixT / 32) {
-        const int cl = (int)meds[mi];
-        const int a = (int)(sst[cl] - s0), len = (int)(sst[cl + 1] - s0) - a;
-        if (len <= 32)
-            warp_seg_sort(buf + a, len);
-        else
-            seg_sort<true>(buf + a, len);
-    }
-    __syncthreads();
-    const int nl = nlong;
-    for (int li = 0; li < nl; ++li) {
-        const int cl = (int)longs[li];
-        const int a = (int)(sst[cl] - s0), e = (int)(sst[cl + 1] - s0);
-        seg_sort<false>(buf + a, e - a);
-    }
-    for (int j = tid; j < n; j += 2 * kFixT) {
-        const int j2 = j + kFixT;
-        const uint32_t i1 = buf[j], i2 = buf[j2 < n ? j2 : j];
-        const Cell c1 = cell_of(pos, np, i1, lattice, N, fN);
-        const Cell c2 = cell_of(pos, np, i2, lattice, N, fN);
-        perm[s0 + j] = i1;
-        if (sfrac) {
-            sfrac[s0 + j] = c1.d[0];
-            sfrac[np + s0 + j] = c1.d[1];
-            sfrac[2 * np + s0 + j] = c1.d[2];
-        }
-        if (j2 < n) {
-            perm[s0 + j2] = i2;
-            if (sfrac) {
-                sfrac[s0 + j2] = c2.d[0];
-                sfrac[np + s0 + j2] = c2.d[1];
-                sfrac[2 * np + s0 + j2] = c2.d[2];
-            }
-        }
-    }
-}
-
-// The runs k_seg_fix could not stage: the same steps on global memory, one
-// block per listed run.
-__global__ void __launch_bounds__(kFixT) k_seg_fix_big(const uint32_t* __restrict__ start, uint32_t* __restrict__ perm,
-                                                       int64_t ncell, const float* __restrict__ pos, int64_t np,
-                                                       bool lattice, int N, FastDiv fN, float* __restrict__ sfrac,
-                                                       const uint32_t* __restrict__ ovf,
-                                                       const uint32_t* __restrict__ novf) {
-    const uint32_t no = *novf;
-    const int tid = threadIdx.x;
-    for (uint32_t bi = blockIdx.x; bi < no; bi += gridDim.x) {
-        const int64_t c0 = (int64_t)ovf[bi] * kFixCells;
-        const int nc = (int)min((int64_t)kFixCells, ncell - c0);
-        for (int cl = tid; cl < nc; cl += kFixT) {
-            const uint32_t a = start[c0 + cl], e = start[c0 + cl + 1];
+    if (big) {  // perm is the list the others are read from: its short segments are put in order here
+        for (int l = tid; l < nc; l += R::T) {
+            const uint32_t a = cst[l], e = cst[l + 1];
             if (e - a <= 1 || e - a > (uint32_t)kSegThread) continue;
             for (uint32_t p = a + 1; p < e; ++p) {
-                const uint32_t v = perm[p];
+                const uint32_t v = seg[p];
                 uint32_t q = p;
-                while (q > a && perm[q - 1] > v) {
-                    perm[q] = perm[q - 1];
-                    --q;
-                }
-                perm[q] = v;
+                for (; q > a && seg[q - 1] > v; --q) seg[q] = seg[q - 1];
+                seg[q] = v;
             }
         }
-        for (int cl = tid >> 5; cl < nc; cl += kFixT / 32) {
-            const uint32_t a = start[c0 + cl], e = start[c0 + cl + 1];
-            if (e - a <= (uint32_t)kSegThread || e - a > (uint32_t)kSegWarp) continue;
-            if (e - a <= 32u)
-                warp_seg_sort(perm + a, (int)(e - a));
-            else
-                seg_sort<true>(perm + a, (int)(e - a));
-        }
         __syncthreads();
-        for (int cl = 0; cl < nc; ++cl) {
-            const uint32_t a = start[c0 + cl], e = start[c0 + cl + 1];
-            if (e - a > (uint32_t)kSegWarp) seg_sort<false>(perm + a, (int)(e - a));
-        }
-        const uint32_t s0 = start[c0], s1 = start[c0 + nc];
-        for (uint32_t j = s0 + tid; j < s1; j += kFixT) write_sorted(perm[j], j, pos, np, lattice, N, fN, perm, sfrac);
-        __syncthreads();
+    }
+    for (int j = tid; j < n; j += R::T) {
+        const float4 q = rec[s0 + j];
+        const uint32_t i = rec_index(q), p = place(rec_cell(q), i);
+        if (!big) perm[p] = i;
+        sfrac[p] = rec_offset(q.x);
+        sfrac[np + p] = rec_offset(q.y);
+        sfrac[2 * np + p] = rec_offset(q.z);
     }
 }
 
@@ -799,35 +829,32 @@ __global__ void k_lpt2_hess_grad(const float* __restrict__ sigma, const float* _
 
 // ============================================================================= host wrappers
 
+int sort_run_log(int64_t ncell) { return ncell >= (int64_t)1 << 21 ? 11 : 9; }
+
 int cell_sort_into(pmr_ctx* c, const float* pos, int64_t np, bool lattice, uint32_t* keys_out, uint32_t* perm,
                    uint32_t* start, float* sfrac) {
     const int N = c->N;
     const int64_t N3 = c->N3;
     const FastDiv fN((uint32_t)N);
-    uint32_t* keys = keys_out ? keys_out : c->keys;
-    uint32_t* rank = c->sort_tmp;  // slot of each particle in its cell, until the scatter
-    PMR_TRY(check_cuda(c, cudaMemsetAsync(c->counts, 0, sizeof(uint32_t) * N3, c->stream), "memset"));
-    PMR_TRY(check_cuda(c, cudaMemsetAsync(c->long_count, 0, sizeof(uint32_t), c->stream), "memset"));
+    const int rs_log = sort_run_log(N3);
+    const int nruns = (int)((N3 + (1 << rs_log) - 1) >> rs_log);
+    uint32_t *cnt = c->run_cnt, *cursor = cnt + nruns * kRunPad, *rstart = cursor + nruns * kRunPad;
+    PMR_TRY(check_cuda(c, cudaMemsetAsync(cnt, 0, sizeof(uint32_t) * nruns * kRunPad, c->stream), "memset"));
     if (np > 0) {
-        k_keys<<<nblocks(np, kT), kT, 0, c->stream>>>(pos, np, lattice, N, fN, keys, c->counts, rank);
-        PMR_TRY(check_launch(c, "keys"));
+        k_run_count<<<nblocks(np, kT * kBinP), kT, 0, c->stream>>>(pos, np, lattice, N, fN, rs_log, keys_out, cnt);
+        PMR_TRY(check_launch(c, "run_count"));
     }
-    const int nb = (int)((N3 + kScanBlock - 1) / kScanBlock);
-    k_scan_reduce<<<nb, kScanT, 0, c->stream>>>(c->counts, N3, c->scan_part);
-    PMR_TRY(check_launch(c, "scan_reduce"));
-    k_scan_part<<<1, kScanPartT, 0, c->stream>>>(c->scan_part, nb, start + N3);
-    PMR_TRY(check_launch(c, "scan_part"));
-    k_scan_apply<<<nb, kScanT, 0, c->stream>>>(c->counts, N3, c->scan_part, start);
-    PMR_TRY(check_launch(c, "scan_apply"));
-    if (np == 0) return PMR_OK;
-    k_scatter<<<nblocks(np, kT), kT, 0, c->stream>>>(keys, rank, np, start, perm);
-    PMR_TRY(check_launch(c, "scatter"));
-    k_seg_fix<<<nblocks(N3, kFixCells), kFixT, 0, c->stream>>>(start, perm, N3, pos, np, lattice, N, fN, sfrac,
-                                                               c->long_list, c->long_count);
-    PMR_TRY(check_launch(c, "seg_fix"));
-    k_seg_fix_big<<<256, kFixT, 0, c->stream>>>(start, perm, N3, pos, np, lattice, N, fN, sfrac, c->long_list,
-                                               c->long_count);
-    return check_launch(c, "seg_fix_big");
+    k_run_scan<<<nblocks(nruns, kScanT), kScanT, 0, c->stream>>>(cnt, nruns, rstart, cursor);
+    PMR_TRY(check_launch(c, "run_scan"));
+    if (np > 0) {
+        k_run_place<<<nblocks(np, kT * kBinP), kT, 0, c->stream>>>(pos, np, lattice, N, fN, rs_log, cursor, c->rec);
+        PMR_TRY(check_launch(c, "run_place"));
+    }
+    if (rs_log == 11)
+        k_run_sort<11><<<nruns, RunCfg<11>::T, 0, c->stream>>>(c->rec, rstart, N3, np, start, perm, sfrac);
+    else
+        k_run_sort<9><<<nruns, RunCfg<9>::T, 0, c->stream>>>(c->rec, rstart, N3, np, start, perm, sfrac);
+    return check_launch(c, "run_sort");
 }
 
 int cell_sort(pmr_ctx* c, const float* pos, int64_t np, bool lattice, uint32_t* keys_out) {
