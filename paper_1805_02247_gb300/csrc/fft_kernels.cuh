@@ -70,8 +70,12 @@ __device__ __forceinline__ float2 root_mul(float2 a) {
         constexpr bool plus_i = (4 * u == R) == INV;
         return plus_i ? make_float2(-a.y, a.x) : make_float2(a.y, -a.x);
     } else {
-        constexpr float c = (float)root_cs(u, R, false), s = (float)root_cs(u, R, true);
-        return cmul(a, make_float2(c, INV ? s : -s));
+        // fused operands spelt out: left to the compiler, the form (and the rounding) would
+        // depend on the constants
+        constexpr float c = (float)root_cs(u, R, false), s = INV ? (float)root_cs(u, R, true) : -(float)root_cs(u, R, true);
+        const float x = fmaf(a.x, c, -__fmul_rn(a.y, s));
+        const float y = INV ? fmaf(a.y, c, __fmul_rn(a.x, s)) : fmaf(a.x, s, __fmul_rn(a.y, c));
+        return make_float2(x, y);
     }
 }
 

@@ -9,7 +9,7 @@ const FFTOps* fft_plans_0(int N) {
         case 12: return Plan<Reg<6, 2>, Reg<6, 1>>::ops();
         case 16: return Plan<Reg<2, 8>, Reg<2, 4>>::ops();
         case 18: return Plan<Reg<6, 3>, Reg<9, 1>>::ops();
-        case 24: return Plan<Reg<4, 6>, Reg<6, 2>>::ops();
+        case 24: return Plan<Reg<4, 6>, Reg<12, 1>>::ops();
         case 32: return Plan<Reg<8, 4>, Reg<4, 4>>::ops();
         case 36: return Plan<Reg<6, 6>, Reg<6, 3>>::ops();
         case 48: return Plan<Reg<12, 4>, Reg<6, 4>>::ops();
