@@ -177,7 +177,8 @@ void for_each_buffer(const pmr_config& cfg, pmr_ctx* c, F alloc) {
 
 size_t lbfgs_bytes(const pmr_config& cfg) {
     const int64_t N = cfg.N, NH = N * N * (N / 2 + 1);
-    return sizeof(double) * 2 * NH * (6 + 2 * (size_t)cfg.lbfgs_m) + sizeof(float2) * NH + sizeof(double) * 80;
+    return sizeof(double) * 2 * NH * (6 + 2 * (size_t)cfg.lbfgs_m) + sizeof(float2) * NH +
+           sizeof(double) * lbfgs_scalars(cfg.lbfgs_m);
 }
 
 void free_all(pmr_ctx* c) {
@@ -524,19 +525,20 @@ int recon_step(pmr_ctx* c, void* s_k_v, const float* data, const pmr_anneal* an,
         L.k = 0;
         L.head = 0;
         PMR_TRY(evaluate(c, s_k, data, an, host, L.gk));
-        PMR_TRY(c64_to_f64(c, s_k, L.x, c->NH));
-        PMR_TRY(c64_to_f64(c, L.gk, L.g, c->NH));
+        PMR_TRY(lbfgs_start(c, s_k));
         L.f = host[0];
         L.have_f = true;
         L.an = *an;
     }
     double sc[3];
+    auto read_scalars = [&](int k) {
+        PMR_TRY(check_cuda(c, cudaMemcpyAsync(sc, L.scal, k * sizeof(double), cudaMemcpyDeviceToHost, c->stream), "rb"));
+        return check_cuda(c, cudaStreamSynchronize(c->stream), "sync");
+    };
     double gd = 0.0;
     if (L.k > 0) {
         PMR_TRY(lbfgs_two_loop(c, L.g, L.S, L.Y, L.k, L.head, L.m, n, L.rho_host.data(), L.d, true));
-        PMR_TRY(dot64(c, L.g, L.d, n, L.scal + 2));
-        PMR_TRY(check_cuda(c, cudaMemcpyAsync(sc, L.scal + 2, sizeof(double), cudaMemcpyDeviceToHost, c->stream), "rb"));
-        PMR_TRY(check_cuda(c, cudaStreamSynchronize(c->stream), "sync"));
+        PMR_TRY(read_scalars(1));
         gd = sc[0];
         if (!(gd < 0)) {
             L.k = 0;
@@ -545,10 +547,8 @@ int recon_step(pmr_ctx* c, void* s_k_v, const float* data, const pmr_anneal* an,
     }
     if (L.k == 0) {
         // first step: -H0 g with H0 = diag(P~ / w), the prior's inverse Hessian
-        PMR_TRY(prior_h0_apply(c, L.d, L.g, -1.0));
-        PMR_TRY(dot64(c, L.g, L.d, n, L.scal + 2));
-        PMR_TRY(check_cuda(c, cudaMemcpyAsync(sc, L.scal + 2, sizeof(double), cudaMemcpyDeviceToHost, c->stream), "rb"));
-        PMR_TRY(check_cuda(c, cudaStreamSynchronize(c->stream), "sync"));
+        PMR_TRY(lbfgs_first_direction(c));
+        PMR_TRY(read_scalars(1));
         gd = sc[0];
         if (!(gd < 0)) return fail(c, PMR_ELINESEARCH, "zero gradient");
     }
@@ -556,8 +556,7 @@ int recon_step(pmr_ctx* c, void* s_k_v, const float* data, const pmr_anneal* an,
     double t = 1.0, fnew = 0.0;
     bool ok = false;
     for (int it = 0; it < 20; ++it) {
-        PMR_TRY(axpy64(c, L.xt, L.d, nullptr, t, n, L.x));
-        PMR_TRY(f64_to_c64(c, L.xt, s_k, c->NH));
+        PMR_TRY(lbfgs_trial(c, t, s_k));
         int rc = evaluate(c, s_k, data, an, host, L.gk);
         if (rc != PMR_OK && rc != PMR_ENAN) return rc;
         if (rc == PMR_OK && host[0] <= L.f + c1 * t * gd) {
@@ -568,18 +567,12 @@ int recon_step(pmr_ctx* c, void* s_k_v, const float* data, const pmr_anneal* an,
         t *= 0.5;
     }
     if (!ok) {
-        PMR_TRY(f64_to_c64(c, L.x, s_k, c->NH));
+        PMR_TRY(lbfgs_restore(c, s_k));
         return fail(c, PMR_ELINESEARCH, "no Armijo step within 20 halvings");
     }
-    PMR_TRY(c64_to_f64(c, L.gk, L.gt, c->NH));
-    // candidate pair s = xt - x (into d), y = gt - g
-    PMR_TRY(axpy64(c, L.d, L.x, nullptr, -1.0, n, L.xt));
-    PMR_TRY(axpy64(c, L.yk, L.g, nullptr, -1.0, n, L.gt));
-    PMR_TRY(dot64(c, L.d, L.yk, n, L.scal + 3));
-    PMR_TRY(dot64(c, L.d, L.d, n, L.scal + 4));
-    PMR_TRY(dot64(c, L.yk, L.yk, n, L.scal + 5));
-    PMR_TRY(check_cuda(c, cudaMemcpyAsync(sc, L.scal + 3, 3 * sizeof(double), cudaMemcpyDeviceToHost, c->stream), "rb"));
-    PMR_TRY(check_cuda(c, cudaStreamSynchronize(c->stream), "sync"));
+    // candidate pair s = xt - x (into d), y = gt - g (into yk)
+    PMR_TRY(lbfgs_candidate(c));
+    PMR_TRY(read_scalars(3));
     if (sc[0] > 1e-10 * std::sqrt(sc[1] * sc[2])) {
         int slot;
         if (L.k < L.m) {
@@ -749,15 +742,7 @@ int pmr_lbfgs_direction(pmr_ctx* c, const double* g, const double* S, const doub
     PMR_TRY(check_ctx(c));
     if (!g || !d || (k > 0 && (!S || !Y))) return fail(c, PMR_EINVAL, "NULL argument");
     if (k < 1 || k > c->cfg.lbfgs_m || n < 1 || n > c->lb.n) return fail(c, PMR_EINVAL, "need 1 <= k <= lbfgs_m, n <= 2 N^2 (N/2+1)");
-    std::vector<double> rho(k), sy(k);
-    for (int t = 0; t < k; ++t) {
-        PMR_TRY(dot64(c, S + (int64_t)t * n, Y + (int64_t)t * n, n, c->red_out + 2));
-        PMR_TRY(check_cuda(c, cudaMemcpyAsync(&sy[t], c->red_out + 2, sizeof(double), cudaMemcpyDeviceToHost, c->stream),
-                           "rb"));
-        PMR_TRY(check_cuda(c, cudaStreamSynchronize(c->stream), "sync"));
-        rho[t] = 1.0 / sy[t];
-    }
-    return lbfgs_two_loop(c, g, S, Y, k, 0, k, n, rho.data(), d, false);
+    return lbfgs_two_loop(c, g, S, Y, k, 0, k, n, nullptr, d, false);
 }
 
 }  // extern "C"

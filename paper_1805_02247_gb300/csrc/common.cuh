@@ -101,6 +101,10 @@ struct FFTPlan {
     float2* twN = nullptr;  // exp(-2 pi i t / N), t < N (device)
 };
 
+constexpr int kLbfgsBlocks = 608;  // 4 blocks on each of 152 SMs
+// doubles of LBFGS::alpha, scal, sums and part together
+inline int64_t lbfgs_scalars(int m) { return m + 8 + (m + 1) + (int64_t)(m + 3) * kLbfgsBlocks; }
+
 // Stored L-BFGS history on the device (float64), oldest first in a ring.
 struct LBFGS {
     int m = 0, k = 0, head = 0;  // capacity, stored pairs, slot of the oldest pair
@@ -114,7 +118,9 @@ struct LBFGS {
     double* S = nullptr;         // [m][n]
     double* Y = nullptr;         // [m][n]
     double* alpha = nullptr;     // [m] first-loop coefficients (device)
-    double* scal = nullptr;      // device scalars (dots)
+    double* scal = nullptr;      // [8] device scalars (dots)
+    double* sums = nullptr;      // [m + 1] dot products of the stored pairs
+    double* part = nullptr;      // [m + 3][kLbfgsBlocks] block partials
     float2* gk = nullptr;        // float32 gradient of the last evaluation (half array)
     std::vector<double> rho_host;  // 1 / (s.y) per slot
     bool have_f = false;
@@ -337,13 +343,11 @@ int lbfgs_alloc(pmr_ctx* c);
 void lbfgs_free(pmr_ctx* c);
 int lbfgs_two_loop(pmr_ctx* c, const double* g, const double* S, const double* Y, int k, int head, int m,
                    int64_t n, const double* rho_host, double* d, bool prior_h0);
-// y = scale * diag(P~ / w) x over the half-array reals (the prior's inverse Hessian)
-int prior_h0_apply(pmr_ctx* c, double* y, const double* x, double scale);
-int dot64(pmr_ctx* c, const double* a, const double* b, int64_t n, double* out_dev);
-int c64_to_f64(pmr_ctx* c, const float2* a, double* out, int64_t nh);
-int f64_to_c64(pmr_ctx* c, const double* a, float2* out, int64_t nh);
-int axpy64(pmr_ctx* c, double* y, const double* x, const double* alpha_dev, double alpha_host, int64_t n,
-           const double* base);
+int lbfgs_first_direction(pmr_ctx* c);             // lb.d = -D g, scal[0] = g.d
+int lbfgs_start(pmr_ctx* c, const float2* s_k);    // lb.x, lb.g from s_k, lb.gk
+int lbfgs_trial(pmr_ctx* c, double t, float2* s_k);  // lb.xt = x + t d and its float32 form
+int lbfgs_restore(pmr_ctx* c, float2* s_k);        // s_k = lb.x
+int lbfgs_candidate(pmr_ctx* c);                   // lb.gt, the pair (lb.d, lb.yk), scal[0..2]
 
 inline unsigned nblocks(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
