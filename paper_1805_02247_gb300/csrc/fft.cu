@@ -101,6 +101,10 @@ int zy_fwd(pmr_ctx* c, const float* const* a, const float* const* b, float ca, f
     }
     z.ca = ca;
     z.cb = cb;
+    if (c->plan.ops->zy) {
+        c->plan.ops->zy(z, n, c->plan.twN, c->stream);
+        return check_launch(c, "zy_fwd");
+    }
     PMR_TRY(launch_z_r2c(c, z, n));
     return launch_col(c, k, y, k, y, n, false);
 }
@@ -116,6 +120,10 @@ int yz_inv(pmr_ctx* c, float2* k, float* const* out, float* const* out2, float s
     }
     z.s1 = s1;
     z.s2 = s2;
+    if (c->plan.ops->yz) {
+        c->plan.ops->yz(z, n, (float)(1.0 / ((double)c->N * c->N)), c->plan.twN, c->stream);
+        return check_launch(c, "yz_inv");
+    }
     PMR_TRY(launch_col(c, k, y, k, y, n, true));
     return launch_z_c2r(c, z, n);
 }

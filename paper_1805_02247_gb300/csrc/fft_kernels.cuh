@@ -297,6 +297,37 @@ __device__ __forceinline__ void four_step_inv(float2 (&v2)[RG::A2][RG::N2], floa
     }
 }
 
+// The two halves of four_step_fwd for a column that lies in shared memory, pitch
+// apart, and transposes in place; the caller separates them with block barriers.
+template <class RG, bool INV>
+__device__ __forceinline__ void plane_first(float2 (&v1)[RG::A1][RG::N1], float2* col, int pitch, const float2* tw,
+                                            int g) {
+#pragma unroll
+    for (int a = 0; a < RG::A1; ++a) {
+        const int n2 = g + RG::G * a;
+        dft_reg<RG::N1, INV>(v1[a]);
+#pragma unroll
+        for (int k1 = 0; k1 < RG::N1; ++k1) {
+            float2 v = v1[a][k1];
+            if (k1 > 0) {
+                float2 w = tw[n2 * k1];
+                if (INV) w.y = -w.y;
+                v = cmul(v, w);
+            }
+            col[(k1 * RG::N2 + n2) * pitch] = v;
+        }
+    }
+}
+template <class RG, bool INV>
+__device__ __forceinline__ void plane_second(float2 (&v2)[RG::A2][RG::N2], const float2* col, int pitch, int g) {
+#pragma unroll
+    for (int a = 0; a < RG::A2; ++a) {
+#pragma unroll
+        for (int n2 = 0; n2 < RG::N2; ++n2) v2[a][n2] = col[((g + RG::G * a) * RG::N2 + n2) * pitch];
+        dft_reg<RG::N2, INV>(v2[a]);
+    }
+}
+
 // rows N2 n1 + n2 of the thread's n2 set
 template <class RG>
 __device__ __forceinline__ void load_n2(float2 (&v1)[RG::A1][RG::N1], const float2* in, int es, bool ok, int g) {
@@ -670,32 +701,19 @@ __device__ __forceinline__ void row_fft(float2* S, const float2* t4, int g, bool
     }
 }
 
-template <class RG>
-__global__ void __launch_bounds__(ZReg<RG>::T) k_z_r2c_reg(const __grid_constant__ ZFwd p, int nrows, const float2* __restrict__ twN) {
-    using Z = ZReg<RG>;
-    constexpr int M = Z::M, N1 = RG::N1, N2 = RG::N2, G = RG::G, A2 = RG::A2;
-    extern __shared__ float2 sm[];
-    float2* tw = sm;               // split table
-    float2* t4 = tw + Z::SPLIT;    // four-step table
-    float2* A = t4 + (M + 1) / 2 * 2;  // [R][PITCH]
-    const int tid = threadIdx.x;
-    const int row0 = blockIdx.x * Z::R;
-    const int rows = min(Z::R, nrows - row0);
-    load_z_tables<Z, RG>(tw, t4, twN);
-    const float* in2 = p.b[blockIdx.y];
-    stage_rows<Z>(A, reinterpret_cast<const float2*>(p.a[blockIdx.y]) + (int64_t)row0 * M, rows,
-                  in2 ? reinterpret_cast<const float2*>(in2) + (int64_t)row0 * M : nullptr, p.ca, p.cb);
-    __syncthreads();
-    int r, g;
-    bool act;
-    z_row<Z>(r, g, act);
-    float2* Ar = A + r * Z::PITCH;
+// Forward transform of the staged row Ar and the real-to-complex split: put(k, X_k) for
+// the thread's k, k = M by thread 0; the row may be overwritten by put. All lanes of
+// the warp take part; act: whether this one stores.
+template <class RG, class Put>
+__device__ __forceinline__ void z_forward_row(float2* Ar, const float2* t4, const float2* tw, int g, bool act, Put put) {
+    constexpr int M = RG::N, N1 = RG::N1, N2 = RG::N2, G = RG::G, A2 = RG::A2;
     float2 v1[RG::A1][N1], v2[A2][N2];
 #pragma unroll
     for (int a = 0; a < RG::A1; ++a)
 #pragma unroll
         for (int n1 = 0; n1 < N1; ++n1) v1[a][n1] = Ar[N2 * n1 + g + G * a];
     row_fft<RG, false>(Ar, t4, g, act, v1, v2);
+    __syncwarp();
     // X_k = E_k + exp(-2 pi i k / N) O_k from Z_k and conj(Z_(M-k)). Z_(M-k) of the
     // thread's k = g + G a + N1 k2 is, for g > 0, element (A2 - 1 - a, N2 - 1 - k2) of
     // thread G - g; for g = 0 one of its own.
@@ -706,11 +724,8 @@ __global__ void __launch_bounds__(ZReg<RG>::T) k_z_r2c_reg(const __grid_constant
         const float2 o = make_float2(0.5f * dd.y, -0.5f * dd.x);  // -i/2 (zk - zc)
         return cadd(e, cmul(tw[kk], o));
     };
-    const int lane = tid & 31;
+    const int lane = threadIdx.x & 31;
     const int src = g == 0 ? lane : lane - g + (G - g);
-    const int row = row0 + r;
-    const bool st = act && r < rows;
-    float2* orow = p.out[blockIdx.y] + (int64_t)row * M;
 #pragma unroll
     for (int a = 0; a < A2; ++a)
 #pragma unroll
@@ -723,34 +738,17 @@ __global__ void __launch_bounds__(ZReg<RG>::T) k_z_r2c_reg(const __grid_constant
             }
             const int k = g + G * a + N1 * k2;
             const float2 x = split(v2[a][k2], zp, k);
-            if (st) orow[k] = x;
+            if (act) put(k, x);
         }
-    if (st && g == 0) p.out[blockIdx.y][(int64_t)nrows * M + row] = split(v2[0][0], v2[0][0], M);
+    if (act && g == 0) put(M, split(v2[0][0], v2[0][0], M));
 }
 
+// Inverse transform of the staged row Ar (its M + 1 values) to the real row at complex
+// offset o of out (and out2).
 template <class RG>
-__global__ void __launch_bounds__(ZReg<RG>::T) k_z_c2r_reg(const __grid_constant__ ZInv p, int nrows, float scale,
-                                                             const float2* __restrict__ twN) {
-    using Z = ZReg<RG>;
-    constexpr int M = Z::M, N = Z::N, N1 = RG::N1, N2 = RG::N2, G = RG::G;
-    extern __shared__ float2 sm[];
-    float2* tw = sm;               // split table
-    float2* t4 = tw + Z::SPLIT;    // four-step table
-    float2* A = t4 + (M + 1) / 2 * 2;  // [R][PITCH]: the M + 1 inputs of each row
-    const int tid = threadIdx.x;
-    const int row0 = blockIdx.x * Z::R;
-    const int rows = min(Z::R, nrows - row0);
-    load_z_tables<Z, RG>(tw, t4, twN);
-    const float2* in = p.in[blockIdx.y];
-    static_assert(Z::R <= Z::T, "one Nyquist value a thread");
-    const float2 nyq = tid < rows ? in[(int64_t)nrows * M + row0 + tid] : make_float2(0.f, 0.f);
-    stage_rows<Z>(A, in + (int64_t)row0 * M, rows, nullptr, 1.f, 0.f);
-    if (tid < Z::R) A[tid * Z::PITCH + M] = nyq;
-    __syncthreads();
-    int r, g;
-    bool act;
-    z_row<Z>(r, g, act);
-    float2* Ar = A + r * Z::PITCH;
+__device__ __forceinline__ void z_inverse_row(float2* Ar, const float2* t4, const float2* tw, int g, bool act, int64_t o,
+                                              float* out, float* out2, float s1, float s2, float scale) {
+    constexpr int M = RG::N, N = 2 * M, N1 = RG::N1, N2 = RG::N2, G = RG::G;
     // z_k = E_k + i O_k with E, O from X_k and conj(X_(M-k))
     float2 v1[RG::A1][N1], v2[RG::A2][N2];
 #pragma unroll
@@ -767,31 +765,215 @@ __global__ void __launch_bounds__(ZReg<RG>::T) k_z_c2r_reg(const __grid_constant
             const float2 e = cscale(cadd(xk, xc), 0.5f);
             float2 w = tw[k];
             w.y = -w.y;  // exp(+2 pi i k / N)
-            const float2 o = cmul(cscale(csub(xk, xc), 0.5f), w);
-            v1[a][n1] = make_float2(e.x - o.y, e.y + o.x);  // e + i o
+            const float2 q = cmul(cscale(csub(xk, xc), 0.5f), w);
+            v1[a][n1] = make_float2(e.x - q.y, e.y + q.x);  // e + i o
         }
     row_fft<RG, true>(Ar, t4, g, act, v1, v2);
     // the row from the four-step's registers straight to global memory
-    if (act && r < rows) {
-        const float sc = scale * 2.0f / (float)N;
-        const int64_t o = (int64_t)(row0 + r) * M;
-        float2* d1 = reinterpret_cast<float2*>(p.out[blockIdx.y]) + o;
-        if (!p.out2[blockIdx.y]) {
+    if (!act) return;
+    const float sc = scale * 2.0f / (float)N;
+    float2* d1 = reinterpret_cast<float2*>(out) + o;
+    if (!out2) {
 #pragma unroll
-            for (int a = 0; a < RG::A2; ++a)
+        for (int a = 0; a < RG::A2; ++a)
 #pragma unroll
-                for (int k2 = 0; k2 < N2; ++k2) d1[g + G * a + N1 * k2] = cscale(v2[a][k2], sc);
-        } else {
-            float2* d2 = reinterpret_cast<float2*>(p.out2[blockIdx.y]) + o;
+            for (int k2 = 0; k2 < N2; ++k2) d1[g + G * a + N1 * k2] = cscale(v2[a][k2], sc);
+    } else {
+        float2* d2 = reinterpret_cast<float2*>(out2) + o;
 #pragma unroll
-            for (int a = 0; a < RG::A2; ++a)
+        for (int a = 0; a < RG::A2; ++a)
 #pragma unroll
-                for (int k2 = 0; k2 < N2; ++k2) {
-                    const float2 v = cscale(v2[a][k2], sc);
-                    d1[g + G * a + N1 * k2] = cscale(v, p.s1);
-                    d2[g + G * a + N1 * k2] = cscale(v, p.s2);
-                }
+            for (int k2 = 0; k2 < N2; ++k2) {
+                const float2 v = cscale(v2[a][k2], sc);
+                d1[g + G * a + N1 * k2] = cscale(v, s1);
+                d2[g + G * a + N1 * k2] = cscale(v, s2);
+            }
+    }
+}
+
+template <class RG>
+__global__ void __launch_bounds__(ZReg<RG>::T) k_z_r2c_reg(const __grid_constant__ ZFwd p, int nrows, const float2* __restrict__ twN) {
+    using Z = ZReg<RG>;
+    constexpr int M = Z::M;
+    extern __shared__ __align__(16) float2 sm[];
+    float2* tw = sm;               // split table
+    float2* t4 = tw + Z::SPLIT;    // four-step table
+    float2* A = t4 + (M + 1) / 2 * 2;  // [R][PITCH]
+    const int tid = threadIdx.x;
+    const int row0 = blockIdx.x * Z::R;
+    const int rows = min(Z::R, nrows - row0);
+    load_z_tables<Z, RG>(tw, t4, twN);
+    const float* in2 = p.b[blockIdx.y];
+    stage_rows<Z>(A, reinterpret_cast<const float2*>(p.a[blockIdx.y]) + (int64_t)row0 * M, rows,
+                  in2 ? reinterpret_cast<const float2*>(in2) + (int64_t)row0 * M : nullptr, p.ca, p.cb);
+    __syncthreads();
+    int r, g;
+    bool act;
+    z_row<Z>(r, g, act);
+    const int row = row0 + r;
+    float2* out = p.out[blockIdx.y];
+    z_forward_row<RG>(A + r * Z::PITCH, t4, tw, g, act && r < rows, [&](int k, float2 x) {
+        out[k < M ? (int64_t)row * M + k : (int64_t)nrows * M + row] = x;
+    });
+}
+
+template <class RG>
+__global__ void __launch_bounds__(ZReg<RG>::T) k_z_c2r_reg(const __grid_constant__ ZInv p, int nrows, float scale,
+                                                             const float2* __restrict__ twN) {
+    using Z = ZReg<RG>;
+    constexpr int M = Z::M;
+    extern __shared__ __align__(16) float2 sm[];
+    float2* tw = sm;               // split table
+    float2* t4 = tw + Z::SPLIT;    // four-step table
+    float2* A = t4 + (M + 1) / 2 * 2;  // [R][PITCH]: the M + 1 inputs of each row
+    const int tid = threadIdx.x;
+    const int row0 = blockIdx.x * Z::R;
+    const int rows = min(Z::R, nrows - row0);
+    load_z_tables<Z, RG>(tw, t4, twN);
+    const float2* in = p.in[blockIdx.y];
+    static_assert(Z::R <= Z::T, "one Nyquist value a thread");
+    const float2 nyq = tid < rows ? in[(int64_t)nrows * M + row0 + tid] : make_float2(0.f, 0.f);
+    stage_rows<Z>(A, in + (int64_t)row0 * M, rows, nullptr, 1.f, 0.f);
+    if (tid < Z::R) A[tid * Z::PITCH + M] = nyq;
+    __syncthreads();
+    int r, g;
+    bool act;
+    z_row<Z>(r, g, act);
+    z_inverse_row<RG>(A + r * Z::PITCH, t4, tw, g, act && r < rows, (int64_t)(row0 + r) * M, p.out[blockIdx.y],
+                      p.out2[blockIdx.y], p.s1, p.s2, scale);
+}
+
+// ----------------------------------------------------------------------------- plane passes
+//
+// Small meshes: an x-plane of the half array (66 KB at N = 128) fits in one block's
+// shared memory, so the z and y passes of a transform run as one kernel, a block per
+// plane: half the launches, which are what a small mesh's transform costs, and one
+// trip through memory instead of two. The row transforms are those of the z pass;
+// the columns lie across the staged rows, one thread group (G threads) a column with
+// the four-step's transpose in the column's own place. The arithmetic of either is
+// that of the separate passes.
+
+template <class RG, class RZ>
+struct PlaneCfg {
+    using Z = ZReg<RZ>;
+    static constexpr int N = RG::N, M = RZ::N, P = M + 1;
+    static constexpr int T = (P * RG::G + 31) / 32 * 32;  // one round of columns
+    static constexpr int ROWS = T / 32 * Z::RW;           // rows a round of the z transforms takes
+    static constexpr size_t smem() {
+        return sizeof(float2) * (size_t)(N + Z::SPLIT + (M + 1) / 2 * 2 + N * Z::PITCH);
+    }
+};
+
+template <class RG, class RZ>
+__global__ void __launch_bounds__(PlaneCfg<RG, RZ>::T) k_zy_plane(const __grid_constant__ ZFwd p,
+                                                                  const float2* __restrict__ twN) {
+    using PC = PlaneCfg<RG, RZ>;
+    using Z = ZReg<RZ>;
+    constexpr int N = PC::N, M = PC::M, P = PC::P, T = PC::T;
+    extern __shared__ __align__(16) float2 sm[];
+    float2* tw = sm;             // N-point table; its first M + 1 entries are the split's
+    float2* t4 = tw + N;         // four-step table of the rows
+    float2* A = t4 + (M + 1) / 2 * 2;
+    const int tid = threadIdx.x, x = blockIdx.x;
+    for (int t = tid; t < N; t += T) tw[t] = twN[t];
+    for (int t = tid; t < M; t += T) t4[t] = twN[2 * (t / RZ::N2) * (t % RZ::N2)];
+    {
+        const float2* s1 = reinterpret_cast<const float2*>(p.a[blockIdx.y]) + (int64_t)x * N * M;
+        const float2* s2 = p.b[blockIdx.y] ? reinterpret_cast<const float2*>(p.b[blockIdx.y]) + (int64_t)x * N * M
+                                           : nullptr;
+#pragma unroll 4
+        for (int t = tid; t < N * M; t += T) {
+            float2 v = s1[t];
+            if (s2) {
+                const float2 w = s2[t];
+                v = make_float2(p.ca * v.x + p.cb * w.x, p.ca * v.y + p.cb * w.y);
+            }
+            const int r = t / M;
+            A[r * Z::PITCH + t - r * M] = v;
         }
+    }
+    __syncthreads();
+    {
+        int r0, g;
+        bool act;
+        z_row<Z>(r0, g, act);
+#pragma unroll 1
+        for (int rr = 0; rr < N; rr += PC::ROWS) {
+            const int r = rr + r0;
+            const bool in = r < N;
+            float2* Ar = A + (in ? r : 0) * Z::PITCH;
+            z_forward_row<RZ>(Ar, t4, tw, g, act && in, [&](int k, float2 v) { Ar[k] = v; });
+        }
+    }
+    __syncthreads();
+    const int c = tid % P, g = tid / P;
+    const bool act = g < RG::G;
+    float2 v1[RG::A1][RG::N1], v2[RG::A2][RG::N2];
+    float2* col = A + c;
+    if (act)
+#pragma unroll
+        for (int a = 0; a < RG::A1; ++a)
+#pragma unroll
+            for (int n1 = 0; n1 < RG::N1; ++n1) v1[a][n1] = col[(RG::N2 * n1 + g + RG::G * a) * Z::PITCH];
+    __syncthreads();
+    if (act) plane_first<RG, false>(v1, col, Z::PITCH, tw, g);
+    __syncthreads();
+    if (!act) return;
+    plane_second<RG, false>(v2, col, Z::PITCH, g);
+    float2* out = p.out[blockIdx.y] + (c < M ? (int64_t)x * N * M + c : (int64_t)N * N * M + (int64_t)x * N);
+    const int es = c < M ? M : 1;
+#pragma unroll
+    for (int a = 0; a < RG::A2; ++a)
+#pragma unroll
+        for (int k2 = 0; k2 < RG::N2; ++k2) out[(g + RG::G * a + RG::N1 * k2) * es] = v2[a][k2];
+}
+
+template <class RG, class RZ>
+__global__ void __launch_bounds__(PlaneCfg<RG, RZ>::T) k_yz_plane(const __grid_constant__ ZInv p, float scale,
+                                                                  const float2* __restrict__ twN) {
+    using PC = PlaneCfg<RG, RZ>;
+    using Z = ZReg<RZ>;
+    constexpr int N = PC::N, M = PC::M, P = PC::P, T = PC::T;
+    extern __shared__ __align__(16) float2 sm[];
+    float2* tw = sm;
+    float2* t4 = tw + N;
+    float2* A = t4 + (M + 1) / 2 * 2;
+    const int tid = threadIdx.x, x = blockIdx.x;
+    const int c = tid % P, g = tid / P;
+    const bool act = g < RG::G;
+    float2 v1[RG::A1][RG::N1], v2[RG::A2][RG::N2];
+    float2* col = A + c;
+    {
+        const float2* in = p.in[blockIdx.y] + (c < M ? (int64_t)x * N * M + c : (int64_t)N * N * M + (int64_t)x * N);
+        const int es = c < M ? M : 1;
+        if (act)
+#pragma unroll
+            for (int a = 0; a < RG::A1; ++a)
+#pragma unroll
+                for (int n1 = 0; n1 < RG::N1; ++n1) v1[a][n1] = in[(RG::N2 * n1 + g + RG::G * a) * es];
+    }
+    for (int t = tid; t < N; t += T) tw[t] = twN[t];
+    for (int t = tid; t < M; t += T) t4[t] = twN[2 * (t / RZ::N2) * (t % RZ::N2)];
+    __syncthreads();
+    if (act) plane_first<RG, true>(v1, col, Z::PITCH, tw, g);
+    __syncthreads();
+    if (act) plane_second<RG, true>(v2, col, Z::PITCH, g);
+    __syncthreads();
+    if (act)
+#pragma unroll
+        for (int a = 0; a < RG::A2; ++a)
+#pragma unroll
+            for (int k2 = 0; k2 < RG::N2; ++k2) col[(g + RG::G * a + RG::N1 * k2) * Z::PITCH] = v2[a][k2];
+    __syncthreads();
+    int r0, gz;
+    bool actz;
+    z_row<Z>(r0, gz, actz);
+#pragma unroll 1
+    for (int rr = 0; rr < N; rr += PC::ROWS) {
+        const int r = rr + r0;
+        const bool in = r < N;
+        z_inverse_row<RZ>(A + (in ? r : 0) * Z::PITCH, t4, tw, gz, actz && in, (int64_t)(x * N + (in ? r : 0)) * M,
+                          p.out[blockIdx.y], p.out2[blockIdx.y], p.s1, p.s2, scale);
     }
 }
 
@@ -804,10 +986,11 @@ struct Plan {
     static constexpr int N = RG::N;
     static_assert(2 * RZ::N == N, "row plan of the same mesh");
     static void z_r2c(const ZFwd& p, int batch, const float2* tw, cudaStream_t s) {
-        k_z_r2c_reg<RZ><<<dim3(nblocks(N * N, Z::R), batch), Z::T, Z::smem(), s>>>(p, N * N, tw);
+        if constexpr (!PLANE) k_z_r2c_reg<RZ><<<dim3(nblocks(N * N, Z::R), batch), Z::T, Z::smem(), s>>>(p, N * N, tw);
     }
     static void z_c2r(const ZInv& p, int batch, float scale, const float2* tw, cudaStream_t s) {
-        k_z_c2r_reg<RZ><<<dim3(nblocks(N * N, Z::R), batch), Z::T, Z::smem(), s>>>(p, N * N, scale, tw);
+        if constexpr (!PLANE)
+            k_z_c2r_reg<RZ><<<dim3(nblocks(N * N, Z::R), batch), Z::T, Z::smem(), s>>>(p, N * N, scale, tw);
     }
     static void col(const float2* in, const Side& si, float2* out, const Side& so, int64_t bs, int batch, bool inv,
                     const float2* tw, cudaStream_t s) {
@@ -817,6 +1000,15 @@ struct Plan {
     // the fused x-pass of a large mesh takes 8 columns a block: 16 would leave one block
     // per SM (512^3 one-to-three: 922 -> 677 us); the plain passes keep 16 (231 against 252 us)
     using RX = Reg<RG::N1, RG::N2, (N >= 384 ? 8 : 16)>;
+    // N <= 128: the y and z passes as one kernel (k_zy_plane, k_yz_plane)
+    using PC = PlaneCfg<RG, RZ>;
+    static constexpr bool PLANE = N <= 128;
+    static void zy(const ZFwd& p, int batch, const float2* tw, cudaStream_t s) {
+        if constexpr (PLANE) k_zy_plane<RG, RZ><<<dim3(N, batch), PC::T, PC::smem(), s>>>(p, tw);
+    }
+    static void yz(const ZInv& p, int batch, float scale, const float2* tw, cudaStream_t s) {
+        if constexpr (PLANE) k_yz_plane<RG, RZ><<<dim3(N, batch), PC::T, PC::smem(), s>>>(p, scale, tw);
+    }
     template <int MODE>
     static void x_mode(const XFused& p, const Side& si, const Side& so, int batch, const float2* tw, cudaStream_t s) {
         k_x_reg<RX, MODE><<<col_grid<RX>(batch), RX::T, RX::smem_x(MODE), s>>>(p, si, so, tw);
@@ -832,8 +1024,13 @@ struct Plan {
         }
     }
     static void each_kernel(void (*set)(void*, const void*, size_t), void* arg) {
-        set(arg, (const void*)k_z_r2c_reg<RZ>, Z::smem());
-        set(arg, (const void*)k_z_c2r_reg<RZ>, Z::smem());
+        if constexpr (PLANE) {
+            set(arg, (const void*)k_zy_plane<RG, RZ>, PC::smem());
+            set(arg, (const void*)k_yz_plane<RG, RZ>, PC::smem());
+        } else {
+            set(arg, (const void*)k_z_r2c_reg<RZ>, Z::smem());
+            set(arg, (const void*)k_z_c2r_reg<RZ>, Z::smem());
+        }
         set(arg, (const void*)k_col_reg<RG, true>, RG::smem_col());
         set(arg, (const void*)k_col_reg<RG, false>, RG::smem_col());
         set(arg, (const void*)k_x_reg<RX, X_1TO1>, RX::smem_x(X_1TO1));
@@ -843,7 +1040,7 @@ struct Plan {
         set(arg, (const void*)k_x_reg<RX, X_NTO1>, RX::smem_x(X_NTO1));
     }
     static const FFTOps* ops() {
-        static const FFTOps o{z_r2c, z_c2r, col, x, each_kernel};
+        static const FFTOps o{z_r2c, z_c2r, PLANE ? zy : nullptr, PLANE ? yz : nullptr, col, x, each_kernel};
         return &o;
     }
 };
