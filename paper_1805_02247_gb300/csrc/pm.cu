@@ -507,6 +507,13 @@ __global__ void __launch_bounds__(RunCfg<RS_LOG>::T, 1024 / RunCfg<RS_LOG>::T)
 // cell in shared memory. Each cell then adds the 2 rows that hold it:
 // rho = U_0(x, y) + U_1(x - 1, y).
 // MMODE 0: unit masses; 1: mass[perm[j]]; 2: masses in sorted order, mass[m][j].
+// Bins with more than kCrowd particles are summed by the whole warp, one after
+// another, if at most kCrowdBins of its 32 are: with more, the lanes side by side are
+// faster (128^3, a collapsed field with rows of such bins: 123 us, the other way 148).
+// In the kernels of the PM path, whose bins hold about one particle, the code for it
+// costs 1.5% (registers) and gains little, so those are built without (CROWD).
+constexpr uint32_t kCrowd = 24;
+constexpr int kCrowdBins = 4;
 template <int NM>
 struct WTile {
     static constexpr int X = 8, Y = NM == 1 ? 16 : 8;
@@ -517,7 +524,7 @@ struct WTile {
     static constexpr size_t smem = sizeof(float) * (2 * NM * X * Y * 32 + 4 * NM * NR);
 };
 
-template <int NM, int MMODE>
+template <int NM, int MMODE, bool CROWD>
 __global__ void __launch_bounds__(WTile<NM>::W * 32, NM == 1 ? 4 : 3) k_paint_wtile(const uint32_t* __restrict__ start,
                                                                      const uint32_t* __restrict__ perm,
                                                                      const float* __restrict__ sfrac,
@@ -574,6 +581,62 @@ __global__ void __launch_bounds__(WTile<NM>::W * 32, NM == 1 ? 4 : 3) k_paint_wt
         load(j, dx, dy, dz, mv);
         acc_v(dx, dy, dz, mv, S, only1);
     };
+    // The sums of a crowded bin by the whole warp, in the same order and arithmetic as by
+    // its one lane: the lanes load 32 particles at a time, and lane 8 m + q adds up corner
+    // q of mass m over them. A lane alone waits for a load per particle, and the warp for
+    // it: clumped particles (128^3, half of them in clumps of 50) 66 -> 49 us.
+    auto crowd = [&](uint32_t s, uint32_t e) {
+        const bool ox = lane & 4, oy = lane & 2, oz = lane & 1;
+        const int mi = lane >> 3;
+        float sum = 0.f;
+        for (uint32_t b = s; b < e; b += 32) {
+            float dx = 0.f, dy = 0.f, dz = 0.f, mv[NM];
+            if (b + lane < e) load(b + lane, dx, dy, dz, mv);
+            const int cnt = (int)min(32u, e - b);
+            for (int i = 0; i < cnt; ++i) {
+                const float x = __shfl_sync(0xffffffffu, dx, i), y = __shfl_sync(0xffffffffu, dy, i);
+                const float z = __shfl_sync(0xffffffffu, dz, i);
+                float w = oz ? z : 1.f - z;
+                if (MMODE) {
+                    float m = __shfl_sync(0xffffffffu, mv[0], i);
+#pragma unroll
+                    for (int k = 1; k < NM; ++k) {
+                        const float mk = __shfl_sync(0xffffffffu, mv[k], i);
+                        if (mi == k) m = mk;
+                    }
+                    w *= m;
+                }
+                const float a = (ox ? x : 1.f - x) * (oy ? y : 1.f - y);
+                sum = fmaf(a, w, sum);
+            }
+        }
+        return sum;
+    };
+    // S of the bins [s, e) of all lanes; the crowded ones first, one after another
+    auto bin_sums = [&](uint32_t s, uint32_t e, float (&S)[2][2][2][NM], bool only1) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+#pragma unroll
+            for (int m = 0; m < NM; ++m) S[q >> 2][(q >> 1) & 1][q & 1][m] = 0.f;
+        uint32_t big = CROWD ? __ballot_sync(0xffffffffu, e - s > kCrowd) : 0u;
+        if (__popc(big) > kCrowdBins) big = 0;  // a dense row: its lanes work side by side
+        while (big) {
+            const int l = __ffs(big) - 1;
+            big &= big - 1;
+            const float sum = crowd(__shfl_sync(0xffffffffu, s, l), __shfl_sync(0xffffffffu, e, l));
+#pragma unroll
+            for (int m = 0; m < NM; ++m)
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    const float v = __shfl_sync(0xffffffffu, sum, 8 * m + q);
+                    if (lane == l) S[q >> 2][(q >> 1) & 1][q & 1][m] = v;
+                }
+            if (lane == l) s = e;
+        }
+        // bins hold about one particle: no unrolled body to skip past
+#pragma unroll 1
+        for (uint32_t j = s; j < e; ++j) acc(j, S, only1);
+    };
 
     // warp w walks the bins of x-row w along y; the next row's bin bounds are
     // loaded before this row's particles
@@ -594,17 +657,21 @@ __global__ void __launch_bounds__(WTile<NM>::W * 32, NM == 1 ? 4 : 3) k_paint_wt
     // neighbour there), one row per lane; only this warp reads them
     float* Hs = Us + 2 * NM * WT::X * WT::Y * 32;  // [4 (ox,oy)][NM][NR]
     static_assert(WTile<NM>::RY <= 32, "one halo row per lane");
-    if (lane < WT::RY) {
+    {
         const int r = bx * WT::RY + lane;
-        const int64_t rb = row_base(r);
-        float H[2][2][2][NM] = {};
-        const uint32_t hs = start[rb + zh], he = start[rb + zh + 1];
-#pragma unroll 1
-        for (uint32_t j = hs; j < he; ++j) acc(j, H, true);
+        uint32_t hs = 0, he = 0;
+        if (lane < WT::RY) {
+            const int64_t rb = row_base(r);
+            hs = start[rb + zh];
+            he = start[rb + zh + 1];
+        }
+        float H[2][2][2][NM];
+        bin_sums(hs, he, H, true);
+        if (lane < WT::RY)
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
+            for (int q = 0; q < 4; ++q)
 #pragma unroll
-            for (int m = 0; m < NM; ++m) Hs[(q * NM + m) * WT::NR + r] = H[q >> 1][q & 1][1][m];
+                for (int m = 0; m < NM; ++m) Hs[(q * NM + m) * WT::NR + r] = H[q >> 1][q & 1][1][m];
     }
     __syncwarp();
     float C[2][NM];   // T_(ox,1) of the previous row
@@ -617,10 +684,8 @@ __global__ void __launch_bounds__(WTile<NM>::W * 32, NM == 1 ? 4 : 3) k_paint_wt
             s_n = start[rb];
             e_n = start[rb + 1];
         }
-        float S[2][2][2][NM] = {};
-        // bins hold about one particle: no unrolled body to skip past
-#pragma unroll 1
-        for (uint32_t j = s; j < e; ++j) acc(j, S, false);
+        float S[2][2][2][NM];
+        bin_sums(s, e, S, false);
 #pragma unroll
         for (int ox = 0; ox < 2; ++ox)
 #pragma unroll
@@ -861,7 +926,7 @@ int cell_sort(pmr_ctx* c, const float* pos, int64_t np, bool lattice, uint32_t* 
     return cell_sort_into(c, pos, np, lattice, keys_out, c->perm, c->cell_start, c->sfrac);
 }
 
-template <int NM, int MMODE>
+template <int NM, int MMODE, bool CROWD>
 int launch_paint_wtile(pmr_ctx* c, const uint32_t* perm, const uint32_t* start, const float* sfrac, const float* mass,
                        int64_t np, float scale, float offset, float* const* rho) {
     using WT = WTile<NM>;
@@ -871,7 +936,7 @@ int launch_paint_wtile(pmr_ctx* c, const uint32_t* perm, const uint32_t* start, 
     static_assert(WTile<1>::smem <= 48 * 1024, "one-mass paint within the default shared-memory limit");
     const int N = c->N;
     const dim3 grid((N + 31) / 32, (N + WT::Y - 1) / WT::Y, (N + WT::X - 1) / WT::X);
-    k_paint_wtile<NM, MMODE><<<grid, WT::W * 32, WT::smem, c->stream>>>(
+    k_paint_wtile<NM, MMODE, CROWD><<<grid, WT::W * 32, WT::smem, c->stream>>>(
         start, perm, sfrac, mass, np, N, scale, offset, rho[0], NM > 1 ? rho[1] : nullptr, NM > 2 ? rho[2] : nullptr);
     return check_launch(c, NM == 1 ? "paint" : "paint3");
 }
@@ -880,10 +945,10 @@ int launch_paint_wtile(pmr_ctx* c, const uint32_t* perm, const uint32_t* start, 
 int paint_with(pmr_ctx* c, const float* pos, int64_t np, bool lattice, const uint32_t* perm, const uint32_t* start,
                const float* sfrac, const float* mass, int nmass, float scale, float offset, float* const* rho) {
     (void)pos;
-    (void)lattice;
     if (!sfrac || nmass != 1) return fail(c, PMR_EINVAL, "paint: one mass and the sort's offsets are required");
-    return mass ? launch_paint_wtile<1, 1>(c, perm, start, sfrac, mass, np, scale, offset, rho)
-                : launch_paint_wtile<1, 0>(c, perm, start, sfrac, nullptr, np, scale, offset, rho);
+    if (mass) return launch_paint_wtile<1, 1, true>(c, perm, start, sfrac, mass, np, scale, offset, rho);
+    return lattice ? launch_paint_wtile<1, 0, false>(c, perm, start, sfrac, nullptr, np, scale, offset, rho)
+                   : launch_paint_wtile<1, 0, true>(c, perm, start, sfrac, nullptr, np, scale, offset, rho);
 }
 
 // Three-mass paint of the lattice particles with their masses first moved into
@@ -896,12 +961,12 @@ int paint3_sorted(pmr_ctx* c, const uint32_t* perm, const uint32_t* start, const
     float* smass = c->F;
     k_permute3<<<nblocks(np, kT), kT, 0, c->stream>>>(perm, mass, np, smass);
     PMR_TRY(check_launch(c, "permute3"));
-    return launch_paint_wtile<3, 2>(c, perm, start, sfrac, smass, np, scale, 0.0f, rho);
+    return launch_paint_wtile<3, 2, false>(c, perm, start, sfrac, smass, np, scale, 0.0f, rho);
 }
 
 int pm_init(pmr_ctx* c) {
     return check_cuda(c,
-                      cudaFuncSetAttribute(k_paint_wtile<3, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                      cudaFuncSetAttribute(k_paint_wtile<3, 2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)WTile<3>::smem),
                       "paint smem attr");
 }
