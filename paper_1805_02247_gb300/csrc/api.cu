@@ -159,7 +159,7 @@ void for_each_buffer(const pmr_config& cfg, pmr_ctx* c, F alloc) {
         alloc((void**)(c ? &c->nn_y : nullptr), sizeof(float) * N3);
         alloc((void**)(c ? &c->nn_m1 : nullptr), sizeof(uint16_t) * 4 * N3);
         alloc((void**)(c ? &c->nn_m2 : nullptr), sizeof(uint8_t) * 4 * N3);
-        if (cfg.head == 1) alloc((void**)(c ? &c->nn_mass : nullptr), sizeof(float) * N3);
+        if (cfg.head == 1) alloc((void**)(c ? &c->nn_mass : nullptr), sizeof(float) * 4 * N3);
     }
     alloc((void**)(c ? &c->cA : nullptr), sizeof(float2) * NH);
     alloc((void**)(c ? &c->cB : nullptr), sizeof(float2) * NH);
@@ -226,7 +226,7 @@ int loss_and_grad_impl(pmr_ctx* c, const float2* s, const float* data, const pmr
     PMR_TRY(pm_forward_impl(c, s));
     PMR_TRY(density_slot(c, c->cfg.nsteps, dfin, c->delta, true));
     PMR_TRY(nn_features(c, c->delta));
-    PMR_TRY(mlp_forward(c, c->feat, c->M, logistic_a(an)));
+    PMR_TRY(mlp_forward(c, c->feat, c->M, logistic_a(an), true));
     PMR_TRY(residual_forward(c, data, an, c->red_out + 1));
     PMR_TRY(prior_value(c, s, c->red_out));
     // adjoint
@@ -406,7 +406,7 @@ int nn_halo_map(pmr_ctx* c, const float* delta, float* mass_out, const pmr_annea
     PMR_TRY(check_ctx(c));
     if (!delta || !mass_out) return fail(c, PMR_EINVAL, "NULL argument");
     PMR_TRY(nn_features(c, delta));
-    return mlp_forward(c, c->feat, mass_out, logistic_a(an));
+    return mlp_forward(c, c->feat, mass_out, logistic_a(an), false);
 }
 
 int nn_halo_map_adjoint(pmr_ctx* c, const float* delta, const float* grad_mass, float* grad_delta,
@@ -415,7 +415,7 @@ int nn_halo_map_adjoint(pmr_ctx* c, const float* delta, const float* grad_mass, 
     if (!delta || !grad_mass || !grad_delta) return fail(c, PMR_EINVAL, "NULL argument");
     PMR_TRY(nn_features(c, delta));
     // the tensor-core backward starts from the forward's saved activations
-    if (c->cfg.nn_path != 2) PMR_TRY(mlp_forward(c, c->feat, c->M, logistic_a(an)));
+    if (c->cfg.nn_path != 2) PMR_TRY(mlp_forward(c, c->feat, c->M, logistic_a(an), true));
     PMR_TRY(mlp_backward(c, c->feat, grad_mass, c->gfeat, logistic_a(an)));
     return features_T(c, c->gfeat, grad_delta);
 }

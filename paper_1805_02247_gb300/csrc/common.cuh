@@ -199,7 +199,7 @@ struct pmr_ctx {
     float* nn_y = nullptr;      // tensor-core network forward, saved per voxel for its backward: y [N3],
     uint16_t* nn_m1 = nullptr;  // layer-1 ReLU mask [4][N3] (16 columns each),
     uint8_t* nn_m2 = nullptr;   // layer-2 ReLU mask [4][N3] (8 columns each)
-    float* nn_mass = nullptr;   // output of the mass network [N3] (two-network head)
+    float* nn_mass = nullptr;   // mass network (two-network head): output [N3], its Jacobian [3][N3]
     float2* cA = nullptr;   // complex work arrays, NH each
     float2* cB = nullptr;
     float2* c3 = nullptr;   // 3 * NH
@@ -311,7 +311,8 @@ int density_slot(pmr_ctx* c, int s, const float* disp, float* delta, bool sort);
 // network (nn.cu) ---------------------------------------------------------------
 int nn_features(pmr_ctx* c, const float* delta);  // -> c->feat
 // a: logistic sharpness of the two-network head (ignored by the softplus head)
-int mlp_forward(pmr_ctx* c, const float* feat, float* M, float a);
+// jac: a backward at the same fields follows
+int mlp_forward(pmr_ctx* c, const float* feat, float* M, float a, bool jac);
 int mlp_backward(pmr_ctx* c, const float* feat, const float* gM, float* gfeat, float a);
 int stencil_transpose(pmr_ctx* c, const float* gv, float* gfeat);
 
@@ -320,11 +321,11 @@ void twopt_free(pmr_ctx* c);
 // network on tcgen05 tensor cores (mlp_tc.cu) -----------------------------------
 int mlp_tc_init(pmr_ctx* c);
 void mlp_tc_free(pmr_ctx* c);
-int mlp_tc_forward(pmr_ctx* c, const float* feat, float* M, int nsplit, float a);
+int mlp_tc_forward(pmr_ctx* c, const float* feat, float* M, int nsplit, float a, bool jac);
 int mlp_tc_backward_gv(pmr_ctx* c, const float* feat, const float* gM, int nsplit, float a);  // -> c->gbox
 int mlp_tc_box_floats(int N);               // size of c->gbox
 // c->gbox (+ the mass network's part) -> input gradient of the three fields
-int stencil_tiles(pmr_ctx* c, const float* feat, const float* gM, float a, float* gfeat);
+int stencil_tiles(pmr_ctx* c, const float* gM, float a, float* gfeat);
 
 // loss (loss.cu) ----------------------------------------------------------------
 int residual_forward(pmr_ctx* c, const float* data, const pmr_anneal* an, double* L_res_dev);

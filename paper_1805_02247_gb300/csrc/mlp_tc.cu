@@ -322,10 +322,14 @@ __device__ __forceinline__ void mass_hidden2(const MassW& W, const float (&h)[20
 
 constexpr int kMassT = 256;
 
-// mass = m, M = M_scale sigmoid(a y) m from the trunk's y
-__global__ void __launch_bounds__(kMassT) k_mass_fwd(const __grid_constant__ MassW W, const float* __restrict__ feat,
+// mass = m, M = M_scale sigmoid(a y) m from the trunk's y; with JAC also the three
+// dm/df_c, J[c][N3], for the backward. The ELU's slope is 1 for x > 0 and e^x =
+// ELU(x) + 1 otherwise, so the Jacobian takes no further exponential.
+template <bool JAC>
+__global__ void __launch_bounds__(kMassT, 4) k_mass_fwd(const __grid_constant__ MassW W, const float* __restrict__ feat,
                                                      const float* __restrict__ y, int64_t N3, float M_scale, float a,
-                                                     float* __restrict__ mass, float* __restrict__ M) {
+                                                     float* __restrict__ mass, float* __restrict__ J,
+                                                     float* __restrict__ M) {
     const int64_t v = (int64_t)blockIdx.x * kMassT + threadIdx.x;
     if (v >= N3) return;
     float h[20], p2[10];
@@ -333,33 +337,27 @@ __global__ void __launch_bounds__(kMassT) k_mass_fwd(const __grid_constant__ Mas
     mass_hidden2(W, h, p2);
     float m = W.w[300];
 #pragma unroll
-    for (int i = 0; i < 10; ++i) m = fmaf(W.w[290 + i], elu_f(p2[i]), m);
-    mass[v] = m;
-    M[v] = M_scale * sigmoidf(a * y[v]) * m;
-}
-
-// g_c += gm dm/df_c at (f0, f1, f2). The ELU's slope is 1 for x > 0 and e^x =
-// ELU(x) + 1 otherwise, so no second exponential is taken.
-__device__ __forceinline__ void mass_grad_add(const MassW& W, float f0, float f1, float f2, float gm, float (&g)[3]) {
-    float h[20], p2[10];
-    mass_hidden1(W, f0, f1, f2, h);
-    mass_hidden2(W, h, p2);
-#pragma unroll
-    for (int i = 0; i < 10; ++i) p2[i] = gm * W.w[290 + i] * (p2[i] > 0.f ? 1.f : expf(p2[i]));
-    float a0 = 0.f, a1 = 0.f, a2 = 0.f;
-#pragma unroll
-    for (int j = 0; j < 20; ++j) {
-        float s = 0.f;
-#pragma unroll
-        for (int i = 0; i < 10; ++i) s = fmaf(W.w[80 + 20 * i + j], p2[i], s);
-        s *= h[j] > 0.f ? 1.f : h[j] + 1.f;
-        a0 = fmaf(W.w[3 * j], s, a0);
-        a1 = fmaf(W.w[3 * j + 1], s, a1);
-        a2 = fmaf(W.w[3 * j + 2], s, a2);
+    for (int i = 0; i < 10; ++i) {
+        const float e = elu_f(p2[i]);
+        m = fmaf(W.w[290 + i], e, m);
+        if (JAC) p2[i] = W.w[290 + i] * (e > 0.f ? 1.f : e + 1.f);  // dm/d(pre-activation)
     }
-    g[0] += a0;
-    g[1] += a1;
-    g[2] += a2;
+    mass[v] = m;
+    if (JAC) {
+        float g[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+        for (int j = 0; j < 20; ++j) {
+            float s = 0.f;
+#pragma unroll
+            for (int i = 0; i < 10; ++i) s = fmaf(W.w[80 + 20 * i + j], p2[i], s);
+            s *= h[j] > 0.f ? 1.f : h[j] + 1.f;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) g[c] = fmaf(W.w[3 * j + c], s, g[c]);
+        }
+#pragma unroll
+        for (int c = 0; c < 3; ++c) J[c * N3 + v] = g[c];
+    }
+    M[v] = M_scale * sigmoidf(a * y[v]) * m;
 }
 
 // Compute warps synchronise among themselves on named barrier 1 (the
@@ -1154,62 +1152,71 @@ TileMap tile_map(const pmr_ctx* c, int* ntiles) {
     return m;
 }
 
-// Candidate (tile, box index) pairs of cell x along one axis: the tiles of the
-// real cells x+1, x, x-1 (periodic), each holding x at box index (p mod TS) + 1 + d;
-// duplicates (the same tile and index reached twice) are dropped.
+// The boxes that hold cell x along one axis of tiles of TS: its own tile's, at box index
+// lx + 1, and on a tile's rim the neighbour's (periodic; the tile of cell x + 1 or x - 1
+// holds x at index 0 or n + 1, n the cells of that tile). A ragged last tile makes its one
+// or two cells rims on both sides; then both neighbours hold them.
+struct AxisBoxes {
+    int t[3], b[3], n;
+};
 template <int TS>
-__device__ __forceinline__ int axis_boxes(int x, int N, int* t_out, int* b_out) {
-    int n = 0;
-#pragma unroll
-    for (int d = 1; d >= -1; --d) {
-        int p = x - d;
-        p = p < 0 ? p + N : (p >= N ? p - N : p);
-        const int t = p / TS, b = p - t * TS + 1 + d;
-        bool dup = false;
-        for (int i = 0; i < n; ++i) dup |= (t_out[i] == t && b_out[i] == b);
-        if (!dup) {
-            t_out[n] = t;
-            b_out[n] = b;
-            ++n;
-        }
-    }
-    return n;
+__device__ __forceinline__ AxisBoxes axis_boxes(int x, int N) {
+    AxisBoxes r;
+    const int xp = x + 1 == N ? 0 : x + 1, xm = x == 0 ? N - 1 : x - 1;
+    const int t = x / TS, tp = xp / TS, tm = xm / TS;
+    // order: the box of the cell below, of the cell itself, of the cell above
+    r.t[0] = tm;
+    r.b[0] = xm - tm * TS + 2;
+    r.t[1] = t;
+    r.b[1] = x - t * TS + 1;
+    r.t[2] = tp;
+    r.b[2] = xp - tp * TS;
+    r.n = (tm != t || r.b[0] != r.b[1] ? 1 : 0) | (tp != t || r.b[2] != r.b[1] ? 2 : 0);  // neighbours present
+    return r;
 }
 
 // What the two-network head adds to the input gradient: the mass network reads
 // the voxel's own fields, M = M_scale sigmoid(a y) m, so with g = gM M_scale
 // sigmoid(a y) the three fields' gradients grow by g dm/df_c.
 struct MassGrad {
-    MassW W;
-    const float *feat, *gM, *y;
+    const float *J, *gM, *y;
     float M_scale, a;
 };
 
 // g_field[c](cell) = sum over the tiles whose box holds the cell, in a fixed
-// order (+ the mass network's part, whose arithmetic hides behind the box loads).
+// order (+ the mass network's part).
 template <bool TWO_NET>
-__global__ void __launch_bounds__(256) k_stencil_tiles(const float* __restrict__ gbox, int N, int nty, int ntz,
-                                                       const __grid_constant__ MassGrad mg,
-                                                       float* __restrict__ gfeat) {
+__global__ void __launch_bounds__(256) k_stencil_tiles(const float* __restrict__ gbox, int N, FastDiv fN, int nty,
+                                                       int ntz, MassGrad mg, float* __restrict__ gfeat) {
     const int64_t N3 = (int64_t)N * N * N;
     const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (v >= N3) return;
-    const int x = (int)(v / ((int64_t)N * N)), y = (int)((v / N) % N), z = (int)(v % N);
-    int tx[3], bx[3], ty[3], by[3], tz[3], bz[3];
-    const int nx = axis_boxes<TX>(x, N, tx, bx), ny = axis_boxes<TY>(y, N, ty, by), nz = axis_boxes<TZ>(z, N, tz, bz);
+    const uint32_t row = fN.div((uint32_t)v);
+    const int z = (int)((uint32_t)v - row * fN.d), x = (int)fN.div(row), y = (int)(row - (uint32_t)x * fN.d);
+    const AxisBoxes ax = axis_boxes<TX>(x, N), ay = axis_boxes<TY>(y, N), az = axis_boxes<TZ>(z, N);
     constexpr int BOX = HX * HY * HZ;
     float acc[3] = {0.f, 0.f, 0.f};
-    for (int i = 0; i < nx; ++i)
-        for (int j = 0; j < ny; ++j)
-            for (int k = 0; k < nz; ++k) {
-                const int64_t tile = ((int64_t)tx[i] * nty + ty[j]) * ntz + tz[k];
-                const float* b = gbox + tile * (3 * BOX) + (bx[i] * HY + by[j]) * HZ + bz[k];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        if (i != 1 && !(ax.n & (i ? 2 : 1))) continue;
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            if (j != 1 && !(ay.n & (j ? 2 : 1))) continue;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                if (k != 1 && !(az.n & (k ? 2 : 1))) continue;
+                const uint32_t tile = ((uint32_t)ax.t[i] * nty + ay.t[j]) * ntz + az.t[k];
+                const float* b = gbox + (int64_t)tile * (3 * BOX) + (ax.b[i] * HY + ay.b[j]) * HZ + az.b[k];
 #pragma unroll
                 for (int c = 0; c < 3; ++c) acc[c] += b[c * BOX];
             }
-    if (TWO_NET)
-        mass_grad_add(mg.W, mg.feat[v], mg.feat[N3 + v], mg.feat[2 * N3 + v],
-                      mg.gM[v] * mg.M_scale * sigmoidf(mg.a * mg.y[v]), acc);
+        }
+    }
+    if (TWO_NET) {
+        const float g = mg.gM[v] * mg.M_scale * sigmoidf(mg.a * mg.y[v]);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) acc[c] = fmaf(g, mg.J[c * N3 + v], acc[c]);
+    }
 #pragma unroll
     for (int c = 0; c < 3; ++c) gfeat[c * N3 + v] = acc[c];
 }
@@ -1251,7 +1258,7 @@ MassW mass_weights(const pmr_ctx* c) {
 }
 
 template <bool BWD, bool BF>
-int launch_tc(pmr_ctx* c, const float* feat, const float* gM, float* M, int nsplit, float a) {
+int launch_tc(pmr_ctx* c, const float* feat, const float* gM, float* M, int nsplit, float a, bool jac) {
     int ntiles = 0;
     TileMap m = tile_map(c, &ntiles);
     const float4* img = reinterpret_cast<const float4*>(BF ? c->tc_img_bf : c->tc_img);
@@ -1273,8 +1280,13 @@ int launch_tc(pmr_ctx* c, const float* feat, const float* gM, float* M, int nspl
                                                      c->cfg.head == 1 ? nullptr : M, sv, c->tc_err, ctl);
         PMR_TRY(check_launch(c, "mlp_tc_fwd"));
         if (c->cfg.head != 1) return PMR_OK;
-        k_mass_fwd<<<nblocks(c->N3, kMassT), kMassT, 0, c->stream>>>(mass_weights(c), feat, c->nn_y, c->N3, Ms, a,
-                                                                     c->nn_mass, M);
+        const unsigned nb = nblocks(c->N3, kMassT);
+        if (jac)
+            k_mass_fwd<true><<<nb, kMassT, 0, c->stream>>>(mass_weights(c), feat, c->nn_y, c->N3, Ms, a, c->nn_mass,
+                                                           c->nn_mass + c->N3, M);
+        else
+            k_mass_fwd<false><<<nb, kMassT, 0, c->stream>>>(mass_weights(c), feat, c->nn_y, c->N3, Ms, a, c->nn_mass,
+                                                            nullptr, M);
         return check_launch(c, "mass_fwd");
     }
     const int grid = std::min(ntiles, c->num_sms);
@@ -1319,27 +1331,28 @@ int mlp_tc_box_floats(int N) {
 
 // input gradient of the three fields from the per-tile box sums of mlp_tc_backward_gv (and,
 // with the two-network head, the mass network's)
-int stencil_tiles(pmr_ctx* c, const float* feat, const float* gM, float a, float* gfeat) {
+int stencil_tiles(pmr_ctx* c, const float* gM, float a, float* gfeat) {
     const int nty = (c->N + TY - 1) / TY, ntz = (c->N + TZ - 1) / TZ;
-    MassGrad mg{};
-    if (c->cfg.head == 1) {
-        mg = MassGrad{mass_weights(c), feat, gM, c->nn_y, (float)c->cfg.M_scale, a};
-        k_stencil_tiles<true><<<nblocks(c->N3, 256), 256, 0, c->stream>>>(c->gbox, c->N, nty, ntz, mg, gfeat);
-    } else {
-        k_stencil_tiles<false><<<nblocks(c->N3, 256), 256, 0, c->stream>>>(c->gbox, c->N, nty, ntz, mg, gfeat);
-    }
+    const FastDiv fN((uint32_t)c->N);
+    const unsigned nb = nblocks(c->N3, 256);
+    if (c->cfg.head == 1)
+        k_stencil_tiles<true><<<nb, 256, 0, c->stream>>>(
+            c->gbox, c->N, fN, nty, ntz, MassGrad{c->nn_mass + c->N3, gM, c->nn_y, (float)c->cfg.M_scale, a}, gfeat);
+    else
+        k_stencil_tiles<false><<<nb, 256, 0, c->stream>>>(c->gbox, c->N, fN, nty, ntz, MassGrad{}, gfeat);
     return check_launch(c, "stencil_tiles");
 }
 
 // nsplit: 3 = TF32 head/tail products (float32 accuracy), 1 = plain TF32, 0 = bf16 operands
-int mlp_tc_forward(pmr_ctx* c, const float* feat, float* M, int nsplit, float a) {
-    return nsplit == 0 ? launch_tc<false, true>(c, feat, nullptr, M, 0, a)
-                       : launch_tc<false, false>(c, feat, nullptr, M, nsplit, a);
+// jac: a backward follows (the mass network's Jacobian is kept for it)
+int mlp_tc_forward(pmr_ctx* c, const float* feat, float* M, int nsplit, float a, bool jac) {
+    return nsplit == 0 ? launch_tc<false, true>(c, feat, nullptr, M, 0, a, jac)
+                       : launch_tc<false, false>(c, feat, nullptr, M, nsplit, a, jac);
 }
 
 int mlp_tc_backward_gv(pmr_ctx* c, const float* feat, const float* gM, int nsplit, float a) {
-    return nsplit == 0 ? launch_tc<true, true>(c, feat, gM, nullptr, 0, a)
-                       : launch_tc<true, false>(c, feat, gM, nullptr, nsplit, a);
+    return nsplit == 0 ? launch_tc<true, true>(c, feat, gM, nullptr, 0, a, false)
+                       : launch_tc<true, false>(c, feat, gM, nullptr, nsplit, a, false);
 }
 
 }  // namespace pmr

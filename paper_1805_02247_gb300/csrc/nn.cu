@@ -208,8 +208,8 @@ int tc_split(const pmr_ctx* c) { return c->cfg.nn_path == 0 ? 3 : (c->cfg.nn_pat
 
 // nn_path 0: tensor cores, 3xTF32 (float32 accuracy); 1: tensor cores, TF32;
 // 2: float32 CUDA cores.
-int mlp_forward(pmr_ctx* c, const float* feat, float* M, float a) {
-    if (c->cfg.nn_path != 2) return mlp_tc_forward(c, feat, M, tc_split(c), a);
+int mlp_forward(pmr_ctx* c, const float* feat, float* M, float a, bool jac) {
+    if (c->cfg.nn_path != 2) return mlp_tc_forward(c, feat, M, tc_split(c), a, jac);
     static_assert(NW == 5661, "weight layout");
     Weights W;
     std::copy(c->W_host.begin(), c->W_host.begin() + (NW + kMassWeights), W.w);
@@ -225,7 +225,7 @@ int stencil_transpose(pmr_ctx* c, const float* gv, float* gfeat) {
 int mlp_backward(pmr_ctx* c, const float* feat, const float* gM, float* gfeat, float a) {
     if (c->cfg.nn_path != 2) {
         PMR_TRY(mlp_tc_backward_gv(c, feat, gM, tc_split(c), a));
-        return stencil_tiles(c, feat, gM, a, gfeat);
+        return stencil_tiles(c, gM, a, gfeat);
     }
     Weights W;
     std::copy(c->W_host.begin(), c->W_host.begin() + (NW + kMassWeights), W.w);
