@@ -297,16 +297,15 @@ int pm_init(pmr_ctx* c);
 int lpt_adjoint(pmr_ctx* c, const float2* s_k, const float* lam_x, const float* lam_p, float2* grad, bool have_H);
 int pm_forward_impl(pmr_ctx* c, const float2* s_k);
 int pm_adjoint_impl(pmr_ctx* c, const float* gfin, float2* grad);  // gfin: gradient w.r.t. the final density
-int density_from(pmr_ctx* c, const float* disp, float* delta);
 // sfrac: the particles' fractional offsets in sorted order, [3][np]
 int cell_sort_into(pmr_ctx* c, const float* pos, int64_t np, bool lattice, uint32_t* keys_out, uint32_t* perm,
-                   uint32_t* start, float* sfrac);
+                   uint32_t* start, float* sfrac, bool counted);
 // sfrac (nullable): the offsets written by the sort that produced perm/start
 int paint_with(pmr_ctx* c, const float* pos, int64_t np, bool lattice, const uint32_t* perm, const uint32_t* start,
                const float* sfrac, const float* mass, int nmass, float scale, float offset, float* const* rho);
-// density of step s's positions; sort == true sorts them into slot s first,
-// otherwise slot s must already hold their sort (from the forward sweep)
-int density_slot(pmr_ctx* c, int s, const float* disp, float* delta, bool sort);
+// sorts step s's positions into slot s and paints their density; stepped: kick_drift
+// produced them just before (and may have counted the runs of their sort)
+int density_slot(pmr_ctx* c, int s, const float* disp, float* delta, bool stepped);
 
 // network (nn.cu) ---------------------------------------------------------------
 int nn_features(pmr_ctx* c, const float* delta);  // -> c->feat

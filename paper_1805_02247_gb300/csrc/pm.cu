@@ -758,8 +758,13 @@ __global__ void k_readout_grad(const float* __restrict__ f, const float* __restr
 // Each thread takes KP particles, blockDim apart, with every load of all of
 // them issued before their arithmetic (more memory requests in flight).
 constexpr int KP = 2;
+// COUNT: it also counts the particles of the next sort's runs (k_run_count's work), one
+// launch less a step. Meshes below 2^21 cells only: beyond, the counting makes this
+// kernel slower by more than the pass it saves (256^3: 250 -> 321 us against 55).
+template <bool COUNT>
 __global__ void k_kick_drift(const float* __restrict__ F, const float* __restrict__ din, float* __restrict__ dout,
-                             float* __restrict__ mom, int64_t np, int N, FastDiv fN, float kick, float drift) {
+                             float* __restrict__ mom, int64_t np, int N, FastDiv fN, float kick, float drift,
+                             int rs_log, uint32_t* __restrict__ cnt) {
     const int64_t i0 = (int64_t)blockIdx.x * blockDim.x * KP + threadIdx.x;
     Cell cl[KP];
     float r[KP][3], p[KP][3], d[KP][3];
@@ -792,12 +797,21 @@ __global__ void k_kick_drift(const float* __restrict__ F, const float* __restric
 #pragma unroll
     for (int u = 0; u < KP; ++u) {
         const int64_t i = i0 + (int64_t)u * blockDim.x;
-        if (i >= np) continue;
+        uint32_t run = kNoRun;
+        if (i < np) {
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            const float pa = p[u][a] + kick * r[u][a];
-            mom[a * np + i] = pa;
-            dout[a * np + i] = d[u][a] + drift * pa;
+            for (int a = 0; a < 3; ++a) {
+                const float pa = p[u][a] + kick * r[u][a];
+                mom[a * np + i] = pa;
+                d[u][a] = d[u][a] + drift * pa;
+                dout[a * np + i] = d[u][a];
+            }
+            if (COUNT) run = key_of(cell_at(d[u], (uint32_t)i, true, N, fN), N) >> rs_log;
+        }
+        if (COUNT) {
+            const uint32_t m = same_run(run);
+            if (run != kNoRun && (m & ((1u << (threadIdx.x & 31)) - 1u)) == 0)
+                atomicAdd(&cnt[run * kRunPad], (uint32_t)__popc(m));
         }
     }
 }
@@ -894,18 +908,31 @@ __global__ void k_lpt2_hess_grad(const float* __restrict__ sigma, const float* _
 
 // ============================================================================= host wrappers
 
+namespace {
+int sort_runs(const pmr_ctx* c) {
+    const int rs_log = sort_run_log(c->N3);
+    return (int)((c->N3 + (1 << rs_log) - 1) >> rs_log);
+}
+// whether kick_drift counts the runs of the sort that follows it
+bool kick_counts(const pmr_ctx* c) { return c->N3 < (int64_t)1 << 21; }
+int clear_run_counts(pmr_ctx* c) {
+    return check_cuda(c, cudaMemsetAsync(c->run_cnt, 0, sizeof(uint32_t) * sort_runs(c) * kRunPad, c->stream), "memset");
+}
+}  // namespace
+
 int sort_run_log(int64_t ncell) { return ncell >= (int64_t)1 << 21 ? 11 : 9; }
 
+// counted: the run counters already hold the counts of pos (kick_drift)
 int cell_sort_into(pmr_ctx* c, const float* pos, int64_t np, bool lattice, uint32_t* keys_out, uint32_t* perm,
-                   uint32_t* start, float* sfrac) {
+                   uint32_t* start, float* sfrac, bool counted) {
     const int N = c->N;
     const int64_t N3 = c->N3;
     const FastDiv fN((uint32_t)N);
     const int rs_log = sort_run_log(N3);
-    const int nruns = (int)((N3 + (1 << rs_log) - 1) >> rs_log);
+    const int nruns = sort_runs(c);
     uint32_t *cnt = c->run_cnt, *cursor = cnt + nruns * kRunPad, *rstart = cursor + nruns * kRunPad;
-    PMR_TRY(check_cuda(c, cudaMemsetAsync(cnt, 0, sizeof(uint32_t) * nruns * kRunPad, c->stream), "memset"));
-    if (np > 0) {
+    if (!counted) PMR_TRY(clear_run_counts(c));
+    if (np > 0 && !counted) {
         k_run_count<<<nblocks(np, kT * kBinP), kT, 0, c->stream>>>(pos, np, lattice, N, fN, rs_log, keys_out, cnt);
         PMR_TRY(check_launch(c, "run_count"));
     }
@@ -923,7 +950,7 @@ int cell_sort_into(pmr_ctx* c, const float* pos, int64_t np, bool lattice, uint3
 }
 
 int cell_sort(pmr_ctx* c, const float* pos, int64_t np, bool lattice, uint32_t* keys_out) {
-    return cell_sort_into(c, pos, np, lattice, keys_out, c->perm, c->cell_start, c->sfrac);
+    return cell_sort_into(c, pos, np, lattice, keys_out, c->perm, c->cell_start, c->sfrac, false);
 }
 
 template <int NM, int MMODE, bool CROWD>
@@ -987,18 +1014,11 @@ int readout_grad(pmr_ctx* c, const float* field, const float* pos, int64_t np, b
     return check_launch(c, "readout_grad");
 }
 
-int density_from(pmr_ctx* c, const float* disp, float* delta) {
-    PMR_TRY(cell_sort(c, disp, c->N3, true, nullptr));
-    float* outs[1] = {delta};
-    // unit-mass particles, one per cell: rho_bar = 1
-    return paint(c, disp, c->N3, true, nullptr, 1, 1.0f, -1.0f, outs);
-}
-
-int density_slot(pmr_ctx* c, int s, const float* disp, float* delta, bool sort) {
+int density_slot(pmr_ctx* c, int s, const float* disp, float* delta, bool stepped) {
     uint32_t* perm = c->perm_all + (int64_t)s * c->N3;
     uint32_t* start = c->start_all + (int64_t)s * (c->N3 + 1);
     float* sfrac = c->sfrac_all + (int64_t)s * 3 * c->N3;
-    if (sort) PMR_TRY(cell_sort_into(c, disp, c->N3, true, nullptr, perm, start, sfrac));
+    PMR_TRY(cell_sort_into(c, disp, c->N3, true, nullptr, perm, start, sfrac, stepped && kick_counts(c)));
     float* outs[1] = {delta};
     return paint_with(c, disp, c->N3, true, perm, start, sfrac, nullptr, 1, 1.0f, -1.0f, outs);
 }
@@ -1083,7 +1103,15 @@ int lpt_adjoint(pmr_ctx* c, const float2* s_k, const float* lam_x, const float* 
 }
 
 int kick_drift(pmr_ctx* c, const float* F, const float* din, float* dout, float* mom, float kick, float drift) {
-    k_kick_drift<<<nblocks(c->N3, kT * KP), kT, 0, c->stream>>>(F, din, dout, mom, c->N3, c->N, FastDiv((uint32_t)c->N), kick, drift);
+    const FastDiv fN((uint32_t)c->N);
+    const int rs_log = sort_run_log(c->N3);
+    const unsigned nb = nblocks(c->N3, kT * KP);
+    if (kick_counts(c)) {
+        PMR_TRY(clear_run_counts(c));
+        k_kick_drift<true><<<nb, kT, 0, c->stream>>>(F, din, dout, mom, c->N3, c->N, fN, kick, drift, rs_log, c->run_cnt);
+    } else {
+        k_kick_drift<false><<<nb, kT, 0, c->stream>>>(F, din, dout, mom, c->N3, c->N, fN, kick, drift, rs_log, nullptr);
+    }
     return check_launch(c, "kick_drift");
 }
 
@@ -1110,7 +1138,7 @@ int pm_forward_impl(pmr_ctx* c, const float2* s_k) {
         float* dout = c->disp + (int64_t)(s + 1) * 3 * N3;
         float* F = c->F_all + (int64_t)s * 3 * N3;  // kept for the adjoint
         float* Fj[3] = {F, F + N3, F + 2 * N3};
-        PMR_TRY(density_slot(c, s, din, c->delta, true));
+        PMR_TRY(density_slot(c, s, din, c->delta, s > 0));
         PMR_TRY(conv_1toN(c, c->delta, Fj, fm, 3));
         PMR_TRY(kick_drift(c, F, din, dout, c->mom, (float)c->kick[s], (float)c->drift[s]));
     }
