@@ -763,8 +763,8 @@ struct LayB {
     static constexpr uint32_t S_GV = S_A4 + L::NP * SZ_A4;
     static constexpr int NTS = 27 * TX * TY * HZ;  // z-folded g_v, Ts[27][TX][TY][HZ]
     static constexpr uint32_t S_TAIL = S_GV + 4 * NTS;
-    // g_y [TM], 8 barriers + TMEM slot
-    static constexpr uint32_t SMEM = S_TAIL + 4 * TM + 80;
+    // 8 barriers + TMEM slot
+    static constexpr uint32_t SMEM = S_TAIL + 80;
     static_assert(SMEM <= 232448, "shared memory budget");
     static_assert(S_B3 % 128 == 0 && S_B4 % 128 == 0 && S_A3 % 128 == 0 && S_A4 % 128 == 0 && S_GV % 16 == 0 &&
                       A3_BUF % 128 == 0 && S_TAIL % 16 == 0,
@@ -787,8 +787,7 @@ __global__ void __launch_bounds__(NTW, 1)
     unsigned char* A4h = sm + B::S_A4;
     unsigned char* A4l = A4h + (L::NP - 1) * B::SZ_A4;
     float* gvs = reinterpret_cast<float*>(sm + B::S_GV);  // Ts[27][TX][TY][HZ]
-    float* gys = reinterpret_cast<float*>(sm + B::S_TAIL);
-    uint64_t* bars = reinterpret_cast<uint64_t*>(gys + TM);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(sm + B::S_TAIL);
     uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + BB_COUNT);
     const float* vec = reinterpret_cast<const float*>(sm + B::S_VEC);
     const float* w3 = vec + 96;
@@ -889,64 +888,53 @@ __global__ void __launch_bounds__(NTW, 1)
             z0 = tz * TZ;
         };
         // saved forward state of a tile, loaded one tile ahead: g_M, y and the mass network's
-        // output of rows tid < TM; the masks of this thread's row and column block
+        // output of this thread's row, the masks of its row and column block
         float L_gm = 0.f, L_y = 0.f, L_mass = 0.f;
         uint32_t L_m1 = 0, L_m2 = 0;
         auto load_saved = [&](int tile) {
             if (tile >= ntiles) return;
             int x0, y0, z0;
             tile_origin(tile, x0, y0, z0);
-            if (tid < TM) {
-                const int gx = x0 + (tid >> 6), gy = y0 + ((tid >> 4) & 3), gz = z0 + (tid & 15);
-                const bool in = gx < N && gy < N && gz < N;
-                const int64_t v = ((int64_t)gx * N + gy) * N + gz;
-                L_gm = in ? gM[v] : 0.f;
-                L_y = in ? sv.y[v] : 0.f;
-                if (TWO_NET) L_mass = in ? sv.mass[v] : 0.f;
-            }
             const int gx = x0 + (row >> 6), gy = y0 + ((row >> 4) & 3), gz = z0 + (row & 15);
             const bool in = gx < N && gy < N && gz < N;
             const int64_t v = ((int64_t)gx * N + gy) * N + gz;
+            L_gm = in ? gM[v] : 0.f;
+            L_y = in ? sv.y[v] : 0.f;
+            if (TWO_NET) L_mass = in ? sv.mass[v] : 0.f;
             L_m1 = in ? sv.m1[cb * N3 + v] : 0u;
             L_m2 = in ? sv.m2[cb * N3 + v] : 0u;
         };
-        // g_y of the loaded tile, A3 = g_a2 = w3 g_y [a2 > 0] into A3 buffer b, arrive on
-        // its "A3 full"
-        auto build_A3 = [&](int tile, int b) {
+        // g_y of the loaded tile's row (each of its four column blocks forms it: a block
+        // barrier to share it cost more), A3 = g_a2 = w3 g_y [a2 > 0] into A3 buffer b,
+        // arrive on its "A3 full"
+        auto build_A3 = [&](int b) {
             unsigned char* A3h = sm + B::S_A3 + (uint32_t)b * B::A3_BUF;
             unsigned char* A3l = A3h + (L::NP - 1) * B::SZ_A3;  // == A3h with one part
-            int x0, y0, z0;
-            tile_origin(tile, x0, y0, z0);
-            if (tid < TM) {
-                const int r = tid;
-                const int gx = x0 + (r >> 6), gy = y0 + ((r >> 4) & 3), gz = z0 + (r & 15);
-                const bool in = gx < N && gy < N && gz < N;
-                const float g = in ? L_gm * M_scale : 0.f;
-                if (TWO_NET) {
-                    // M = M_scale p m: dM/dy = M_scale m a p (1 - p)
-                    const float p = sigmoidf(a * L_y);
-                    gys[r] = g * L_mass * a * p * (1.f - p);
-                } else {
-                    gys[r] = g * sigmoidf(L_y);
-                }
+            float g = L_gm * M_scale;  // 0 outside the mesh
+            if (TWO_NET) {
+                // M = M_scale p m: dM/dy = M_scale m a p (1 - p)
+                const float p = sigmoidf(a * L_y);
+                g = g * L_mass * a * p * (1.f - p);
+            } else {
+                g = g * sigmoidf(L_y);
             }
-            nbar_sync(NT);
-            {
-                const float g = gys[row];
-                float v[8];
+            float v[8];
 #pragma unroll
-                for (int j = 0; j < 8; ++j) v[j] = ((L_m2 >> j) & 1u) ? w3[8 * cb + j] * g : 0.f;
-                put8<BF>(A3h, A3l, row, 8 * cb, v);
-            }
+            for (int j = 0; j < 8; ++j) v[j] = ((L_m2 >> j) & 1u) ? w3[8 * cb + j] * g : 0.f;
+            put8<BF>(A3h, A3l, row, 8 * cb, v);
             fence_async_smem();
             tc_fence_before();
             mbar_arrive(bars + BB_A3 + b);
         };
         // bounded wait on a commit barrier, agreed by all compute threads (the box
         // sums below keep named barriers in the loop)
-        auto wait_commit = [&](int bar, uint32_t& ph, int bit) {
-            const bool got = nbar_and(NT, mbar_wait(bars + bar, (ph >> bit) & 1u, ctl.wait_limit));
+        auto poll = [&](int bar, uint32_t& ph, int bit) {
+            const bool got = mbar_wait(bars + bar, (ph >> bit) & 1u, ctl.wait_limit);
             ph ^= 1u << bit;
+            return got;
+        };
+        auto agree = [&](bool got) {
+            got = nbar_and(NT, got);
             if (got) tc_fence_after();
             return got;
         };
@@ -1050,32 +1038,33 @@ __global__ void __launch_bounds__(NTW, 1)
         uint32_t m1_cur = 0;
         load_saved(tile);
         if (tile < ntiles) {
-            build_A3(tile, 0);
+            build_A3(0);
             m1_cur = L_m1;
             load_saved(tile + gridDim.x);
         }
         for (int it = 0; tile < ntiles; tile += gridDim.x, ++it, last_it = it) {
             const int b = it & 1, nxt = tile + gridDim.x;
-            // (1) the previous tile's layer-1 input gradient (frees A4)
-            if (prev >= 0 && !(ok = wait_commit(BB_D4 + (b ^ 1), ph4, b ^ 1))) break;
-            // (2) this tile's layer-2 input gradient -> A4
-            if (!(ok = wait_commit(BB_D3 + b, ph3, b))) break;
+            // (1) the previous tile's layer-1 input gradient (frees A4) and this tile's
+            //     layer-2 input gradient -> A4
+            bool got = prev < 0 || poll(BB_D4 + (b ^ 1), ph4, b ^ 1);
+            got = poll(BB_D3 + b, ph3, b) && got;
+            if (!(ok = agree(got))) break;
             epilogue3(b, m1_cur);
-            // (3) the next tile's A3 (its buffer's previous MMA3 and D3 reads are done)
+            // (2) the next tile's A3 (its buffer's previous MMA3 and D3 reads are done)
             uint32_t m1_nxt = 0;
             if (nxt < ntiles) {
-                build_A3(nxt, b ^ 1);
+                build_A3(b ^ 1);
                 m1_nxt = L_m1;
                 load_saved(nxt + gridDim.x);
             }
-            // (4) g_v and box sums of the previous tile while this tile's MMA4 runs
+            // (3) g_v and box sums of the previous tile while this tile's MMA4 runs
             if (prev >= 0) epilogue4(prev, b ^ 1);
             m1_cur = m1_nxt;
             prev = tile;
         }
         if (ok && prev >= 0) {
             const int b = (last_it - 1) & 1;
-            if ((ok = wait_commit(BB_D4 + b, ph4, b))) epilogue4(prev, b);
+            if ((ok = agree(poll(BB_D4 + b, ph4, b)))) epilogue4(prev, b);
         }
         if (!ok && tid == 0) atomicExch(err, 1);
     }
