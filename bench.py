@@ -54,24 +54,25 @@ def algorithmic(name: str, N: int):
     N3 = N**3
     NH = N * N * (N // 2 + 1)
     table = {
-        "z_r2c": ("bytes", 4 * N3 + 8 * NH),
-        "z_c2r": ("bytes", 8 * NH + 4 * N3),
-        "col_pass": ("bytes", 16 * NH),
+        # _2, _3: two or three arrays in one launch; zy_fwd and yz_inv do both passes of a plane
+        **{k + sfx: ("bytes", b * m) for m, sfx in ((1, ""), (2, "_2"), (3, "_3"))
+           for k, b in (("z_r2c", 4 * N3 + 8 * NH), ("z_c2r", 8 * NH + 4 * N3), ("col_pass", 16 * NH),
+                        ("zy_fwd", 4 * N3 + 8 * NH), ("yz_inv", 8 * NH + 4 * N3))},
+        "x_conv_1_2": ("bytes", 32 * NH),
         "x_conv_1": ("bytes", 16 * NH), "x_conv_3": ("bytes", 32 * NH), "x_conv_in3": ("bytes", 32 * NH),
         "x_fwd_1": ("bytes", 16 * NH), "x_fwd_in3": ("bytes", 32 * NH),
         "x_inv_3": ("bytes", 32 * NH), "x_inv_1": ("bytes", 16 * NH),
         "paint": ("bytes", (12 + 4 + 4) * N3),         # sorted offsets, bin starts -> density
         "paint3": ("bytes", (12 + 4 + 12 + 12) * N3),  # sorted offsets, starts, 3 sorted masses -> 3 meshes
         "permute3": ("bytes", (4 + 12 + 12) * N3),  # perm, 3 masses -> 3 masses in sorted order
-        "seg_fix": ("bytes", (4 + 8 + 12 + 12) * N3),  # starts, perm r/w, positions -> sorted offsets
-        "scan_reduce": ("bytes", 4 * N3),
-        "scan_apply": ("bytes", 8 * N3),
         "kick_drift": ("bytes", (12 + 12 + 24 + 12) * N3),  # F, disp in, mom r/w, disp out
         "adj_direct": ("bytes", (12 + 12 + 24 + 24) * N3),  # F, disp, lam_x r/w, lam_p r/w
         "readout_grad": ("bytes", (4 + 12 + 24) * N3),
         "adj_readout_direct": ("bytes", (4 + 12 + 12 + 12 + 24 + 24) * N3),  # G, disp_s, F, disp_s-1, lam_x, lam_p r/w
-        "keys": ("bytes", (12 + 4 + 4 + 8) * N3),  # positions -> keys, ranks; counts r/w
-        "scatter": ("bytes", (4 + 4 + 4 + 4) * N3),  # keys, ranks, starts -> perm
+        "run_count": ("bytes", 12 * N3),              # positions
+        "run_place": ("bytes", (12 + 16) * N3),       # positions -> 16-byte binned particles
+        "run_sort": ("bytes", (16 + 16 + 4) * N3),    # binned particles -> perm, sorted offsets; starts
+        "mass_fwd": ("bytes", (12 + 4 + 4 + 12 + 4) * N3),  # fields, y -> mass, its Jacobian, M
         "stencil_T": ("bytes", (81 + 3) * 4 * N3),
         "mlp_fwd": ("flops", MLP_FWD_FLOP * N3),
         "mlp_bwd": ("flops", MLP_BWD_FLOP * N3),
@@ -80,8 +81,6 @@ def algorithmic(name: str, N: int):
         "lpt2_source": ("bytes", (24 + 4) * N3),
         "lpt2_finish": ("bytes", (12 + 12 + 12 + 12) * N3),
         "lpt2_hess_grad": ("bytes", (4 + 12 + 24) * N3),
-        "za_finish": ("bytes", (12 + 12 + 12) * N3),
-        "za_adj_combine": ("bytes", (12 + 12 + 12) * N3),
         "prior": ("bytes", 8 * NH),
         "prior_grad": ("bytes", 8 * NH * 2),
         "log_residual": ("bytes", (4 + 4 + 4) * N3),
@@ -95,17 +94,9 @@ def algorithmic(name: str, N: int):
 # kernels on this workload, one evaluation's launches averaged; kernels changed
 # since their counters were taken have no entry. Valid for N = 256 only.
 TRAFFIC_256 = {
-    "x_conv_3": 68.6e6 + 141.2e6,
     "adj_readout_direct": 1035.9e6 + 373.0e6,  # mean of the 9 + 1 launches of its two forms
-    "x_conv_in3": 203.0e6 + 43.5e6,
-    "col_pass": 67.7e6 + 8.9e6,
-    "z_c2r": 67.7e6 + 17.1e6,
-    "z_r2c": 67.1e6 + 15.2e6,
     "kick_drift": 605.8e6 + 360.3e6,
-    "seg_fix": 336.5e6 + 223.5e6,
-    "keys": 268.6e6 + 152.1e6,
     "permute3": 269.3e6 + 167.0e6,
-    "scatter": 201.8e6 + 43.6e6,
 }
 
 

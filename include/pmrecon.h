@@ -120,7 +120,7 @@ int pmr_destroy(pmr_ctx* ctx);
 int pmr_set_stream(pmr_ctx* ctx, void* stream);
 
 /* Serving aid (no counterpart in the paper): with enable != 0, the launches of
- * one loss_and_grad evaluation (the ~480 kernels of the ICs, PM steps, network,
+ * one loss_and_grad evaluation (the ~230 kernels of the ICs, PM steps, network,
  * loss and adjoint) are captured once into a CUDA graph and replayed as one
  * graph launch for every later evaluation with the same s_k, data, anneal
  * parameters and gradient buffer (recon_step's line-search trials, repeated

@@ -39,19 +39,24 @@ Lay lay_own(int N) { return Lay{N * (N / 2), N / 2, N * N * (N / 2), N, 1}; }
 Side side_y(const Lay& l) { return Side{l.sx, l.sy, l.n0, l.nx, l.ny}; }
 Side side_x(const Lay& l) { return Side{l.sy, l.sx, l.n0, l.ny, l.nx}; }
 
+// launches of one, two or three arrays go by names of their own: their algorithmic bytes differ
+const char* by_batch(int batch, const char* one, const char* two, const char* three) {
+    return batch == 1 ? one : batch == 2 ? two : three;
+}
+
 int launch_z_r2c(pmr_ctx* c, const ZFwd& p, int batch) {
     c->plan.ops->z_r2c(p, batch, c->plan.twN, c->stream);
-    return check_launch(c, "z_r2c");
+    return check_launch(c, by_batch(batch, "z_r2c", "z_r2c_2", "z_r2c_3"));
 }
 
 int launch_z_c2r(pmr_ctx* c, const ZInv& p, int batch) {
     c->plan.ops->z_c2r(p, batch, (float)(1.0 / ((double)c->N * c->N)), c->plan.twN, c->stream);
-    return check_launch(c, "z_c2r");
+    return check_launch(c, by_batch(batch, "z_c2r", "z_c2r_2", "z_c2r_3"));
 }
 
 int launch_col(pmr_ctx* c, const float2* in, const Side& si, float2* out, const Side& so, int batch, bool inv) {
     c->plan.ops->col(in, si, out, so, c->NH, batch, inv, c->plan.twN, c->stream);
-    return check_launch(c, "col_pass");
+    return check_launch(c, by_batch(batch, "col_pass", "col_pass_2", "col_pass_3"));
 }
 
 // batch: the number of one-input, one-output transforms (p.in[b] -> p.out[b], p.mul[0])
@@ -67,7 +72,7 @@ int launch_x_fused(pmr_ctx* c, const XFused& p, const Lay& li, const Lay& lo, in
     static const char* names[2][2][4] = {
         {{"x_mul_1", "x_mul_1", "x_mul_2", "x_mul_3"}, {"x_inv_1", "x_inv_1", "x_inv_2", "x_inv_3"}},
         {{"x_fwd_1", "x_fwd_1", "x_fwd_2", "x_fwd_3"}, {"x_conv_1", "x_conv_1", "x_conv_2", "x_conv_3"}}};
-    const char* nm = names[p.fwd ? 1 : 0][p.inv ? 1 : 0][width];
+    const char* nm = batch > 1 ? "x_conv_1_2" : names[p.fwd ? 1 : 0][p.inv ? 1 : 0][width];
     return check_launch(c, p.nin > 1 ? (p.inv ? "x_conv_in3" : "x_fwd_in3") : nm);
 }
 
@@ -103,7 +108,7 @@ int zy_fwd(pmr_ctx* c, const float* const* a, const float* const* b, float ca, f
     z.cb = cb;
     if (c->plan.ops->zy) {
         c->plan.ops->zy(z, n, c->plan.twN, c->stream);
-        return check_launch(c, "zy_fwd");
+        return check_launch(c, by_batch(n, "zy_fwd", "zy_fwd_2", "zy_fwd_3"));
     }
     PMR_TRY(launch_z_r2c(c, z, n));
     return launch_col(c, k, y, k, y, n, false);
@@ -122,7 +127,7 @@ int yz_inv(pmr_ctx* c, float2* k, float* const* out, float* const* out2, float s
     z.s2 = s2;
     if (c->plan.ops->yz) {
         c->plan.ops->yz(z, n, (float)(1.0 / ((double)c->N * c->N)), c->plan.twN, c->stream);
-        return check_launch(c, "yz_inv");
+        return check_launch(c, by_batch(n, "yz_inv", "yz_inv_2", "yz_inv_3"));
     }
     PMR_TRY(launch_col(c, k, y, k, y, n, true));
     return launch_z_c2r(c, z, n);
